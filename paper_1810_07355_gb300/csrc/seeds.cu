@@ -5,12 +5,16 @@
 //           Lea and Flood 2014) that starts at global_seed + q * 2^32; a draw z
 //           maps to floor(z * n / 2^64) and repeats are redrawn.
 //   pivot:  the n_seed nearest (distance, id) of the P pivots floor(t * n / P).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <climits>
 #include <cmath>
 
 #include "common.cuh"
 #include "warp_sort.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace onng {
 namespace {
@@ -56,31 +60,54 @@ __global__ void seeds_random_kernel(unsigned long long global_seed, int64_t nq, 
         o[t] = chosen[t];
 }
 
-// Nearest-pivot seeds, one CTA per kPivQ queries.  The CTA walks the pivots in
-// tiles of kPivT: each tile (in chunks of kPivD coordinates) and the CTA's
-// queries are staged in shared memory, and thread (i, j) accumulates the
-// squared distances of query i to pivots j, j + 16, j + 32, j + 48 of the tile
-// by direct difference in float32, coordinate by coordinate.  After each tile a
-// warp per query folds the tile's 64 (distance, pivot index) keys into the
-// query's sorted list of its 64 best so far.  Only keys below the list's
-// n_seed-th take part: a few of them are inserted one at a time; when many
-// qualify (the first tiles) the list and the tile are bitonic-sorted together.
-// Every pivot row is read once per CTA instead of once per query, and shared
-// memory (33 KB, so that five CTAs share an SM) does not grow with the pivot
-// count.
-constexpr int kPivQ = 16;
-constexpr int kPivT = 64;
-constexpr int kPivD = 64;
+// Nearest-pivot seeds.  A CTA owns kPivQ queries and a share of the pivots, walked
+// in tiles of kPivT; the S CTAs of a cluster share the queries and split the pivots.
+//
+// Distances: the squared differences are added coordinate by coordinate in float32,
+// one chain per (query, pivot) pair.  What bounds the pass is the float32 pipe (a
+// subtraction and a multiply-add per pair and coordinate), so a thread keeps 4
+// queries x 8 pivots in registers and the two pivots of a pair share each packed
+// instruction (add.f32x2, fma.f32x2: the same rounding per half as the scalar
+// forms).  The operands come from shared memory in the layout the packed form
+// wants: pivots coordinate-major (a 16-byte read is two pairs), queries negated and
+// duplicated; per coordinate 4 reads feed 32 packed instructions.  Chunks of kPivD
+// coordinates are double-buffered: the next chunk's global loads are issued before
+// the arithmetic of the present one and stored to shared memory after it.
+//
+// Selection: after each tile a warp per query folds its kPivT (distance bits, pivot
+// index) keys into the query's sorted list.  Keys below the list's m-th take part;
+// when many do (the first tile), the m-th smallest of the 32 lanes' minima bounds
+// the tile's own m-th smallest key first, which leaves little more than m keys to
+// insert.  At the end the CTAs of the cluster merge their lists over distributed
+// shared memory, each for its share of the queries.
+constexpr int kPivQ = 32;
+constexpr int kPivT = 256;
+constexpr int kPivD = 16;
 constexpr int kPivThreads = 256;
-constexpr int kPivMinCta = 5;
-constexpr int kPivRow = kPivD + 4;  // padded tile row: conflict-free 16-byte reads
-constexpr int kPivInsertMax = 16;   // at most this many qualifying keys: insert one by one
+constexpr int kPivMinCta = 2;
+constexpr int kPivRow = kPivT + 4;  // 4 rows apart is 16 banks apart: conflict-free transposing stores
+constexpr int kPivMaxCluster = 8;
+constexpr int kPivInsertMax = 16;  // more qualifying keys than this are thinned out before insertion
 constexpr unsigned long long kNoKey = ~0ull;
 
-size_t pivot_smem_bytes()
+struct PivSmem {
+    float ts[2][kPivD][kPivRow];   // a chunk of the tile's pivots, coordinate-major
+    float2 qs[2][kPivD][kPivQ];    // the queries' chunk, negated, each value twice
+    float dist[kPivQ][kPivRow];    // the tile's squared distances
+    unsigned long long best[kPivQ][kMaxSeed];
+};
+
+__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b)
 {
-    return sizeof(float) * ((size_t)kPivQ * kPivD + (size_t)kPivT * kPivRow + (size_t)kPivQ * kPivT) +
-           sizeof(unsigned long long) * (size_t)kPivQ * kMaxSeed;
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
 }
 
 // Inserts `key` (warp-uniform, absent from the list) into the ascending list
@@ -96,123 +123,241 @@ __device__ __forceinline__ void list_insert(unsigned long long (&b)[2], unsigned
     b[1] = e1 < pos ? b[1] : (e1 == pos ? key : (lane == 0 ? last0 : up1));
 }
 
+// The list's m-th key (kNoKey while it holds fewer).
+__device__ __forceinline__ unsigned long long list_mth(const unsigned long long (&b)[2], int m)
+{
+    return __shfl_sync(0xffffffffu, m > 32 ? b[1] : b[0], (m - 1) & 31);
+}
+
+// Inserts the lanes' keys `v` that lie below kth (the list's m-th key), updating both.
+__device__ __forceinline__ void list_fold(unsigned long long (&b)[2], unsigned long long v, unsigned long long &kth, int m,
+                                          int lane)
+{
+    unsigned in = __ballot_sync(0xffffffffu, v < kth);
+    while (in) {
+        const int src = __ffs(in) - 1;
+        in &= in - 1;
+        const unsigned long long key = __shfl_sync(0xffffffffu, v, src);
+        if (key < kth) {
+            list_insert(b, key, lane);
+            kth = list_mth(b, m);
+        }
+    }
+}
+
 __global__ void __launch_bounds__(kPivThreads, kPivMinCta)
     seeds_pivot_kernel(const float *__restrict__ X, int64_t n, int d, const float *__restrict__ Q, int64_t nq, int P,
                        int n_seed, int32_t *__restrict__ out)
 {
-    extern __shared__ __align__(16) float psm[];
-    float *qs = psm;                     // [kPivQ][kPivD]
-    float *ts = qs + kPivQ * kPivD;      // [kPivT][kPivRow]
-    float *dist = ts + kPivT * kPivRow;  // [kPivQ][kPivT]: the tile's squared distances
-    unsigned long long *best = reinterpret_cast<unsigned long long *>(dist + kPivQ * kPivT);  // [kPivQ][kMaxSeed]
-    const int tid = threadIdx.x;
-    const int qi = tid >> 4, pj = tid & 15;
-    const int warp = tid >> 5, lane = tid & 31;
+    extern __shared__ __align__(16) unsigned char piv_raw[];
+    PivSmem &sm = *reinterpret_cast<PivSmem *>(piv_raw);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int S = (int)gridDim.y, rank = (int)blockIdx.y;  // the cluster spans the grid's y
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t q0 = (int64_t)blockIdx.x * kPivQ;
+    const int nrow = nq - q0 < kPivQ ? (int)(nq - q0) : kPivQ;
     const int d4 = d >> 2;
     const int m = n_seed < P ? n_seed : P;
+    const int tb = (int)((int64_t)P * rank / S), te = (int)((int64_t)P * (rank + 1) / S);  // this CTA's pivots
     for (int e = tid; e < kPivQ * kMaxSeed; e += kPivThreads)
-        best[e] = kNoKey;
-    for (int t0 = 0; t0 < P; t0 += kPivT) {
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int c0 = 0; c0 < d4; c0 += kPivD / 4) {
-            __syncthreads();
-            // stage the queries' and the tile's coordinates c0*4 .. c0*4 + kPivD (zero past d)
-            for (int e = tid; e < kPivQ * (kPivD / 4); e += kPivThreads) {
-                const int r = e / (kPivD / 4), c = e % (kPivD / 4);
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (q0 + r < nq && c0 + c < d4)
-                    v = __ldg(reinterpret_cast<const float4 *>(Q + (q0 + r) * d) + c0 + c);
-                reinterpret_cast<float4 *>(qs + r * kPivD)[c] = v;
-            }
-            for (int e = tid; e < kPivT * (kPivD / 4); e += kPivThreads) {
-                const int r = e / (kPivD / 4), c = e % (kPivD / 4);
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (t0 + r < P && c0 + c < d4) {
-                    const int64_t id = (int64_t)(t0 + r) * n / P;
-                    v = __ldg(reinterpret_cast<const float4 *>(X + id * d) + c0 + c);
-                }
-                reinterpret_cast<float4 *>(ts + r * kPivRow)[c] = v;
-            }
-            __syncthreads();
-            const float4 *qr = reinterpret_cast<const float4 *>(qs + qi * kPivD);
-#pragma unroll 4
-            for (int c = 0; c < kPivD / 4; ++c) {
-                const float4 a = qr[c];
+        sm.best[e / kMaxSeed][e % kMaxSeed] = kNoKey;
+
+    // staging: thread -> 4 pivot quads (row and quad of the chunk) and, below 128, one query quad
+    const int prow = warp * 16 + (lane >> 1), pc = lane & 1;
+    const int qrow = tid & 31, qc = tid >> 5;
+    float4 pv[4], qv;
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto fetch = [&](int t0, int c0) {
 #pragma unroll
-                for (int mm = 0; mm < 4; ++mm) {
-                    const float4 b = reinterpret_cast<const float4 *>(ts + (pj + 16 * mm) * kPivRow)[c];
-                    float u = a.x - b.x;
-                    acc[mm] = fmaf(u, u, acc[mm]);
-                    u = a.y - b.y;
-                    acc[mm] = fmaf(u, u, acc[mm]);
-                    u = a.z - b.z;
-                    acc[mm] = fmaf(u, u, acc[mm]);
-                    u = a.w - b.w;
-                    acc[mm] = fmaf(u, u, acc[mm]);
-                }
+        for (int h = 0; h < 2; ++h) {
+            const int t = t0 + prow + 128 * h;
+            const float4 *row = reinterpret_cast<const float4 *>(X + (int64_t)t * n / P * d);
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                const int c = c0 + 2 * g + pc;
+                pv[2 * h + g] = t < te && c < d4 ? __ldg(row + c) : zero4;
             }
         }
-#pragma unroll
-        for (int mm = 0; mm < 4; ++mm)
-            dist[qi * kPivT + pj + 16 * mm] = acc[mm];
-        __syncthreads();
-        // fold the tile into each query's best list: keys (distance bits, pivot
-        // index) order as (distance, index) for non-negative distances; NaN
-        // distances (non-finite input) are never taken
-        for (int i = warp; i < kPivQ; i += kPivThreads / 32) {
-            unsigned long long *bl = best + i * kMaxSeed;
-            unsigned long long b[2], v[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int t = t0 + lane + 32 * h;
-                const float dv = dist[i * kPivT + lane + 32 * h];
-                v[h] = (t < P && !isnan(dv)) ? pack_key(dv, t) : kNoKey;
-                b[h] = bl[lane + 32 * h];
-            }
-            const bool hi = m > 32;  // the n_seed-th key sits in b[1]
-            unsigned long long kth = __shfl_sync(0xffffffffu, hi ? b[1] : b[0], (m - 1) & 31);
-            unsigned in0 = __ballot_sync(0xffffffffu, v[0] < kth);
-            unsigned in1 = __ballot_sync(0xffffffffu, v[1] < kth);
-            const int cnt = __popc(in0) + __popc(in1);
-            if (cnt > kPivInsertMax) {
-                unsigned long long s[4] = {b[0], b[1], v[0], v[1]};
-                warp_bitonic_sort<4>(s, lane);
-                b[0] = s[0];
-                b[1] = s[1];
-            } else {
-                while (in0 | in1) {
-                    const bool first = in0 != 0;
-                    const unsigned mk = first ? in0 : in1;
-                    const int src = __ffs(mk) - 1;
-                    if (first)
-                        in0 &= in0 - 1;
-                    else
-                        in1 &= in1 - 1;
-                    const unsigned long long key = __shfl_sync(0xffffffffu, first ? v[0] : v[1], src);
-                    if (key < kth) {
-                        list_insert(b, key, lane);
-                        kth = __shfl_sync(0xffffffffu, hi ? b[1] : b[0], (m - 1) & 31);
-                    }
-                }
-            }
-            if (cnt) {
-                bl[lane] = b[0];
-                bl[32 + lane] = b[1];
-            }
-            __syncwarp();
+        if (tid < 4 * kPivQ) {
+            const int c = c0 + qc;
+            qv = qrow < nrow && c < d4 ? __ldg(reinterpret_cast<const float4 *>(Q + (q0 + qrow) * d) + c) : zero4;
         }
+    };
+    auto store = [&](int b) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int g = 0; g < 2; ++g) {
+                const float4 v = pv[2 * h + g];
+                const int c = (2 * g + pc) * 4, r = prow + 128 * h;
+                sm.ts[b][c][r] = v.x;
+                sm.ts[b][c + 1][r] = v.y;
+                sm.ts[b][c + 2][r] = v.z;
+                sm.ts[b][c + 3][r] = v.w;
+            }
+        if (tid < 4 * kPivQ) {
+            sm.qs[b][qc * 4][qrow] = make_float2(-qv.x, -qv.x);
+            sm.qs[b][qc * 4 + 1][qrow] = make_float2(-qv.y, -qv.y);
+            sm.qs[b][qc * 4 + 2][qrow] = make_float2(-qv.z, -qv.z);
+            sm.qs[b][qc * 4 + 3][qrow] = make_float2(-qv.w, -qv.w);
+        }
+    };
+    // arithmetic: warp -> 16 queries x 64 pivots, lane -> 4 queries x (4 + 4) pivots
+    const int tq = (warp & 1) * 16 + (lane & 3) * 4, tp = (warp >> 1) * 64 + (lane >> 2) * 4;
+    const bool busy = (warp & 1) * 16 < nrow;
+    unsigned long long acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            acc[i][j] = 0ull;
+
+    int b = 0;
+    if (tb < te) {
+        fetch(tb, 0);
+        store(0);
     }
     __syncthreads();
-    for (int i = warp; i < kPivQ; i += kPivThreads / 32) {
-        const int64_t q = q0 + i;
-        if (q >= nq)
-            break;
-        for (int r = lane; r < n_seed; r += 32) {
-            const unsigned long long key = r < m ? best[i * kMaxSeed + r] : kNoKey;
-            out[q * n_seed + r] = key == kNoKey ? -1 : (int32_t)((int64_t)(unsigned)(key & 0xFFFFFFFFull) * n / P);
+    for (int t0 = tb; t0 < te; t0 += kPivT) {
+        for (int c0 = 0; c0 < d4; c0 += kPivD / 4) {
+            const bool last = c0 + kPivD / 4 >= d4;
+            const int nt = last ? t0 + kPivT : t0, nc = last ? 0 : c0 + kPivD / 4;
+            if (nt < te)
+                fetch(nt, nc);
+            if (busy) {
+#pragma unroll
+                for (int c = 0; c < kPivD; ++c) {
+                    const ulonglong2 x0 = *reinterpret_cast<const ulonglong2 *>(&sm.ts[b][c][tp]);
+                    const ulonglong2 x1 = *reinterpret_cast<const ulonglong2 *>(&sm.ts[b][c][tp + 32]);
+                    const ulonglong2 q01 = *reinterpret_cast<const ulonglong2 *>(&sm.qs[b][c][tq]);
+                    const ulonglong2 q23 = *reinterpret_cast<const ulonglong2 *>(&sm.qs[b][c][tq + 2]);
+                    const unsigned long long qq[4] = {q01.x, q01.y, q23.x, q23.y};
+                    const unsigned long long xx[4] = {x0.x, x0.y, x1.x, x1.y};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const unsigned long long u = add_f32x2(xx[j], qq[i]);
+                            acc[i][j] = fma_f32x2(u, u, acc[i][j]);
+                        }
+                }
+            }
+            if (last) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    *reinterpret_cast<ulonglong2 *>(&sm.dist[tq + i][tp]) = make_ulonglong2(acc[i][0], acc[i][1]);
+                    *reinterpret_cast<ulonglong2 *>(&sm.dist[tq + i][tp + 32]) = make_ulonglong2(acc[i][2], acc[i][3]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        acc[i][j] = 0ull;
+                }
+            }
+            if (nt < te)
+                store(b ^ 1);
+            __syncthreads();
+            b ^= 1;
+        }
+        // fold the tile into each query's list; keys order as (distance, pivot index)
+        // and NaN distances (non-finite input) are never taken
+        for (int i = warp; i < nrow; i += kPivThreads / 32) {
+            unsigned long long v[8], l[2] = {sm.best[i][lane], sm.best[i][32 + lane]};
+            unsigned long long kth = list_mth(l, m);
+            int cnt = 0;
+#pragma unroll
+            for (int h = 0; h < 8; ++h) {
+                const int t = t0 + h * 32 + lane;
+                const float dv = sm.dist[i][h * 32 + lane];
+                v[h] = (t < te && !isnan(dv)) ? pack_key(dv, t) : kNoKey;
+                cnt += __popc(__ballot_sync(0xffffffffu, v[h] < kth));
+            }
+            if (!cnt)
+                continue;
+            if (cnt > kPivInsertMax && m > 32) {
+#pragma unroll
+                for (int h = 0; h < 8; h += 2) {
+                    unsigned long long s[4] = {l[0], l[1], v[h], v[h + 1]};
+                    warp_bitonic_sort<4>(s, lane);
+                    l[0] = s[0];
+                    l[1] = s[1];
+                }
+            } else {
+                if (cnt > kPivInsertMax) {
+                    unsigned long long mn[1] = {v[0]};
+#pragma unroll
+                    for (int h = 1; h < 8; ++h)
+                        mn[0] = v[h] < mn[0] ? v[h] : mn[0];
+                    warp_bitonic_sort<1>(mn, lane);
+                    const unsigned long long lim = __shfl_sync(0xffffffffu, mn[0], m - 1);
+#pragma unroll
+                    for (int h = 0; h < 8; ++h)
+                        v[h] = v[h] <= lim ? v[h] : kNoKey;
+                }
+#pragma unroll
+                for (int h = 0; h < 8; ++h)
+                    list_fold(l, v[h], kth, m, lane);
+            }
+            sm.best[i][lane] = l[0];
+            sm.best[i][32 + lane] = l[1];
         }
     }
+    if (S > 1)
+        cluster.sync();
+    else
+        __syncthreads();
+    // merge the cluster's lists: this CTA takes the queries rank, rank + S, ...
+    for (int i = rank + S * warp; i < nrow; i += S * (kPivThreads / 32)) {
+        unsigned long long l[2] = {sm.best[i][lane], sm.best[i][32 + lane]};
+        if (S > 1) {
+            unsigned long long kth = list_mth(l, m);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                if (h * 32 >= m)
+                    break;
+                unsigned long long o[kPivMaxCluster];  // the other lists' keys, all loads in flight
+#pragma unroll
+                for (int r = 0; r < kPivMaxCluster; ++r) {
+                    o[r] = kNoKey;
+                    if (r < S && r != rank)
+                        o[r] = cluster.map_shared_rank(&sm.best[0][0], r)[i * kMaxSeed + h * 32 + lane];
+                }
+#pragma unroll
+                for (int r = 0; r < kPivMaxCluster; ++r)
+                    list_fold(l, o[r], kth, m, lane);
+            }
+        }
+        const int64_t q = q0 + i;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = h * 32 + lane;
+            const unsigned long long key = r < m ? l[h] : kNoKey;
+            if (r < n_seed)
+                out[q * n_seed + r] = key == kNoKey ? -1 : (int32_t)((int64_t)(unsigned)(key & 0xFFFFFFFFull) * n / P);
+        }
+    }
+    if (S > 1)
+        cluster.sync();  // no CTA leaves while another reads its lists
+}
+
+// CTAs per cluster: how often the pivots of a query block are split.  The grid's time
+// is waves x (tiles per CTA + the fixed selection and merge work, about 64
+// coordinates' worth of a tile); the smallest split with the least such time is taken.
+int pivot_split(int64_t nq, int P, int d, int64_t slots)
+{
+    const int64_t blocks = (nq + kPivQ - 1) / kPivQ;
+    int best = 1;
+    int64_t best_cost = INT64_MAX;
+    for (int s = 1; s <= kPivMaxCluster; s *= 2) {
+        if (s > 1 && P / s < 64)
+            break;
+        const int64_t share = (P + s - 1) / s;
+        const int64_t waves = (blocks * s + slots - 1) / slots;
+        const int64_t cost = waves * ((share + kPivT - 1) / kPivT * d + 64) * 256 + share;
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = s;
+        }
+    }
+    return best;
 }
 }  // namespace
 }  // namespace onng
@@ -257,11 +402,24 @@ extern "C" int onng_seeds_pivot(const float *X, int64_t n, int32_t d, const floa
     ONNG_REQUIRE(X && Q && out, ONNG_E_INVAL, "onng_seeds_pivot: NULL pointer");
     ONNG_REQUIRE(aligned16(X) && aligned16(Q), ONNG_E_INVAL, "onng_seeds_pivot: X and Q must be 16-byte aligned");
     const int P = (int)std::min<int64_t>(n_pivot, n);
-    const size_t sm = pivot_smem_bytes();
+    const size_t sm = sizeof(PivSmem);
     ONNG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void *>(seeds_pivot_kernel),
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),
                   "onng_seeds_pivot: smem attribute");
-    seeds_pivot_kernel<<<(unsigned)((nq + kPivQ - 1) / kPivQ), kPivThreads, sm, to_cuda(stream)>>>(X, n, d, Q, nq, P,
-                                                                                                  n_seed, out);
+    const int S = pivot_split(nq, P, d, (int64_t)num_sms() * kPivMinCta);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((nq + kPivQ - 1) / kPivQ), (unsigned)S);
+    cfg.blockDim = dim3(kPivThreads);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = to_cuda(stream);
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 1;
+    attr.val.clusterDim.y = (unsigned)S;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    ONNG_CUDA_TRY(cudaLaunchKernelEx(&cfg, seeds_pivot_kernel, X, n, (int)d, Q, nq, P, (int)n_seed, out),
+                  "onng_seeds_pivot");
     return check_launch("onng_seeds_pivot");
 }

@@ -63,7 +63,7 @@ int onng_version(void);
  * self_offset + r and that id is excluded (a duplicate point with another id is
  * still a neighbour).  k <= 256.  Rows with fewer than k candidates are padded
  * with -1 / +inf.  Three sweeps over the base: byte-valued inputs (integers
- * 0-255) at d = 64 / 128 on the tensor cores, ranked exactly (the lists are
+ * 0-255) at d = 32 .. 128 on the tensor cores, ranked exactly (the lists are
  * written as ranked); other non-integer inputs at d >= 32 on the tensor cores
  * with both sets centred on the base mean and split into bfloat16 hi + lo (dot
  * products to about 2^-16 |q| |x|), and the rest by a float32 SIMT sweep

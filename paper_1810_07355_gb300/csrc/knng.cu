@@ -18,7 +18,7 @@
 // Integer-valued inputs whose squared norms stay below 2^23 are ranked exactly:
 // every product, partial sum and the expanded form are exact in float32.
 //
-// Which sweep runs (onng_knn): byte-valued inputs at d = 64 / 128 take the
+// Which sweep runs (onng_knn): byte-valued inputs at d = 32 .. 128 take the
 // tensor cores exactly (knn_tc_kernel); other non-integer inputs at d >= 32 take
 // the tensor cores in a split bfloat16 form (knn_tcs_kernel) whose survivors are
 // rescored; everything else, and problems smaller than one tile, the SIMT sweep.
@@ -35,7 +35,7 @@
 namespace onng {
 namespace {
 
-constexpr int BM = 128, BN = 128, BK = 16, NT = 256;
+constexpr int BN = 128, BK = 16, NT = 256;
 constexpr int BUF = 256;  // candidate buffer entries per row (>= 2 * BN)
 constexpr unsigned long long EMPTY_KEY = 0x7F800000FFFFFFFFull;  // (+inf, id -1)
 
@@ -64,118 +64,346 @@ __global__ void norms_kernel(const float *__restrict__ X, int64_t n, int d, floa
         out[row] = s;
 }
 
-// Loads a BK-wide slab of 128 rows (rows >= nrows and dims >= d read as 0) and
-// stores it transposed: S[k][m].
-__device__ __forceinline__ void load_slab(const float *__restrict__ M, int64_t row0, int64_t nrows, int d, int k0,
-                                          float (*S)[BM + 4], int tid)
+// Compact warp sorts for the sweeps' epilogues: the stage loops run at run
+// time (only the loop over a lane's registers is unrolled), so the code stays
+// small enough for the instruction cache next to the epilogue's hot loop.
+// Element e = i * 32 + lane lives in v[i] of lane `lane`.
+
+// compare-exchange of registers i and i ^ JR (partners 32 JR elements apart),
+// ascending where bit `size` of the element index is clear
+template <int JR, int N>
+__device__ __forceinline__ void cas_regs(unsigned long long (&v)[N], int lane, int size)
 {
 #pragma unroll
-    for (int t = 0; t < (BM * BK / 4) / NT; ++t) {
-        const int f = tid + t * NT;
-        const int m = f >> 2;
-        const int kq = (f & 3) << 2;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (row0 + m < nrows && k0 + kq < d)
-            v = __ldg(reinterpret_cast<const float4 *>(M + (row0 + m) * d + k0 + kq));
-        S[kq + 0][m] = v.x;
-        S[kq + 1][m] = v.y;
-        S[kq + 2][m] = v.z;
-        S[kq + 3][m] = v.w;
+    for (int i = 0; i < N; ++i) {
+        const int ii = i ^ JR;
+        if (ii > i) {
+            const bool asc = (((i << 5) | lane) & size) == 0;
+            const unsigned long long a = v[i], b = v[ii];
+            const bool sw = asc ? (a > b) : (a < b);
+            v[i] = sw ? b : a;
+            v[ii] = sw ? a : b;
+        }
     }
 }
 
-template <int KC, int NBUF = BUF>
-__device__ void merge_row(int r, int64_t grow, unsigned long long *__restrict__ best, unsigned long long *__restrict__ buf,
-                          float *s_thr, int *s_cnt, int lane)
+// one bitonic step at distance j elements for sequences of length `size`
+template <int N>
+__device__ __forceinline__ void bitonic_step(unsigned long long (&v)[N], int lane, int size, int j)
 {
-    static_assert(KC + NBUF <= 512, "merge sorts 512 keys");
-    const int cnt = s_cnt[r];
-    unsigned long long v[16];
+    if (j >= 32) {
+        const int jr = j >> 5;
+        if constexpr (N >= 2)
+            if (jr == 1)
+                cas_regs<1>(v, lane, size);
+        if constexpr (N >= 4)
+            if (jr == 2)
+                cas_regs<2>(v, lane, size);
+        if constexpr (N >= 8)
+            if (jr == 4)
+                cas_regs<4>(v, lane, size);
+    } else {
+        const bool lower = (lane & j) == 0;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const int e = i * 32 + lane;
-        if (e < KC)
-            v[i] = best[grow * KC + e];
-        else if (e - KC < cnt)
-            v[i] = buf[grow * NBUF + (e - KC)];
-        else
-            v[i] = EMPTY_KEY;
-    }
-    warp_bitonic_sort<16>(v, lane);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const int e = i * 32 + lane;
-        if (e < KC)
-            best[grow * KC + e] = v[i];
-    }
-    const unsigned long long last = __shfl_sync(0xffffffffu, v[(KC - 1) >> 5], (KC - 1) & 31);
-    __syncwarp();
-    if (lane == 0) {
-        s_thr[r] = key_dist(last);
-        s_cnt[r] = 0;
+        for (int i = 0; i < N; ++i) {
+            const bool asc = (((i << 5) | lane) & size) == 0;
+            const unsigned long long o = __shfl_xor_sync(0xffffffffu, v[i], j);
+            const bool take_min = lower == asc;
+            v[i] = take_min ? (o < v[i] ? o : v[i]) : (o > v[i] ? o : v[i]);
+        }
     }
 }
 
+// ascending sort of 32 N keys
+template <int N> __device__ void warp_sort_compact(unsigned long long (&v)[N], int lane)
+{
+    static_assert(N == 1 || N == 2 || N == 4 || N == 8, "N in {1, 2, 4, 8}");
+#pragma unroll 1
+    for (int size = 2; size <= 32 * N; size <<= 1)
+#pragma unroll 1
+        for (int j = size >> 1; j > 0; j >>= 1)
+            bitonic_step<N>(v, lane, size, j);
+}
+
+// ascending merge of a bitonic sequence of 32 N keys (one bitonic merge pass with
+// every element's direction ascending)
+template <int N> __device__ void warp_merge_compact(unsigned long long (&v)[N], int lane)
+{
+#pragma unroll 1
+    for (int j = 16 * N; j > 0; j >>= 1)
+        bitonic_step<N>(v, lane, 64 * N, j);
+}
+
+// The warp merges row gr's cnt buffered keys into its sorted best list of KC
+// keys and returns the new threshold: the distance of list entry kth (< KC).
 template <int KC>
+__device__ __noinline__ float merge_row(int64_t gr, int cnt, int kth, unsigned long long *__restrict__ best,
+                                           const unsigned long long *__restrict__ buf, int lane)
+{
+    static_assert(KC <= BUF && BUF == 256, "the buffer sort holds 256 keys");
+    constexpr int PB = KC / 32;
+    unsigned long long a[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int e = i * 32 + lane;
+        a[i] = e < cnt ? buf[gr * BUF + e] : EMPTY_KEY;
+    }
+    // sort the smallest power-of-two prefix holding the cnt keys (the rest is +inf)
+    if (cnt <= 64) {
+        unsigned long long t[2] = {a[0], a[1]};
+        warp_sort_compact<2>(t, lane);
+        a[0] = t[0];
+        a[1] = t[1];
+    } else if (cnt <= 128) {
+        unsigned long long t[4] = {a[0], a[1], a[2], a[3]};
+        warp_sort_compact<4>(t, lane);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            a[i] = t[i];
+    } else {
+        warp_sort_compact<8>(a, lane);
+    }
+    unsigned long long bv[PB], m[PB];
+#pragma unroll
+    for (int i = 0; i < PB; ++i)
+        bv[i] = best[gr * KC + i * 32 + lane];
+    // half-cleaner of (a[0 .. KC), reversed best): the smaller of each pair is a
+    // bitonic sequence holding the KC smallest keys
+#pragma unroll
+    for (int i = 0; i < PB; ++i) {
+        const unsigned long long br = __shfl_sync(0xffffffffu, bv[PB - 1 - i], 31 - lane);
+        m[i] = a[i] < br ? a[i] : br;
+    }
+    warp_merge_compact<PB>(m, lane);
+#pragma unroll
+    for (int i = 0; i < PB; ++i)
+        best[gr * KC + i * 32 + lane] = m[i];
+    unsigned long long kv = m[0];
+#pragma unroll
+    for (int i = 1; i < PB; ++i)
+        kv = (kth >> 5) == i ? m[i] : kv;
+    return key_dist(__shfl_sync(0xffffffffu, kv, kth & 31));
+}
+
+// Which share of a sweep a CTA takes.  The row blocks below `main` are swept by gm
+// CTAs each (share g of gm), the later ones by gt: these would fill only part of the
+// last wave, so more CTAs share each of them.  Every share keeps a best list and a
+// candidate buffer of its own: lists g < gm of all rows, then lists gm .. gt - 1 of
+// the rows from block `main` on.
+struct Shares {
+    int64_t main, blocks;  // row blocks swept by gm CTAs each; all row blocks
+    int gm, gt;
+    __host__ __device__ int64_t ctas() const { return main * gm + (blocks - main) * gt; }
+};
+
+struct Share {
+    int64_t block;
+    int g, G;
+};
+
+__device__ __forceinline__ Share my_share(const Shares &sh, int64_t cta)
+{
+    const int64_t cut = sh.main * sh.gm;
+    if (cta < cut)
+        return {cta / sh.gm, (int)(cta % sh.gm), sh.gm};
+    return {sh.main + (cta - cut) / sh.gt, (int)((cta - cut) % sh.gt), sh.gt};
+}
+
+// first key (or buffer entry) of list g of row 0 if it existed: rows are `per` entries
+// apart; `rows` is the block size
+__host__ __device__ __forceinline__ int64_t list_base(const Shares &sh, int g, int64_t nq, int rows, int64_t per)
+{
+    if (g < sh.gm)
+        return (int64_t)g * nq * per;
+    const int64_t first = sh.main * rows, tail = nq - first;
+    return ((int64_t)sh.gm * nq + (int64_t)(g - sh.gm) * tail - first) * per;
+}
+
+// lists (of one row each) that the shares of nq rows need
+int64_t list_rows(const Shares &sh, int64_t nq, int rows)
+{
+    const int64_t tail = sh.blocks > sh.main ? nq - sh.main * rows : 0;
+    return (int64_t)sh.gm * nq + (int64_t)(sh.gt - sh.gm) * tail;
+}
+
+// The shares of a sweep of `tiles` base tiles by `blocks` row blocks on `slots`
+// resident CTAs: whole waves unsplit (gm CTAs a block), and the blocks of the last,
+// partial wave split so that its CTAs end soonest (ceil(blocks gt / slots) rounds of
+// tiles / gt tiles, plus about `warm` tiles' worth for every further list: its
+// threshold starts from nothing).
+Shares plan_shares(int64_t blocks, int64_t tiles, int64_t slots, int gm, int64_t warm)
+{
+    Shares sh;
+    sh.blocks = blocks;
+    sh.gm = sh.gt = gm;
+    sh.main = blocks * gm / slots * slots / gm;
+    const int64_t rem = blocks - sh.main;
+    if (rem == 0)
+        return sh;
+    int64_t best = INT64_MAX;
+    for (int64_t g = gm; g <= std::min<int64_t>(std::max<int64_t>(tiles / 4, gm), std::max<int64_t>(8, slots / rem)); ++g) {
+        const int64_t cost = (rem * g + slots - 1) / slots * ((tiles + g - 1) / g + warm);
+        if (cost < best) {
+            best = cost;
+            sh.gt = (int)g;
+        }
+    }
+    if (sh.gt == gm)
+        sh.main = blocks;
+    return sh;
+}
+
+constexpr int kSweepSms = 152;  // SMs the sweeps are planned for
+
+__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// The float32 sweep.  RM rows x 8 columns per thread, so a row block is BM = 16 RM
+// rows: sweeps of fewer than 128 queries take the smallest block that holds them
+// (the arithmetic of padding rows is what bounded them).  The products use packed
+// multiply-adds (two columns per instruction, the same rounding as the scalar form);
+// the queries sit in shared memory duplicated, the base tile coordinate-major, and the
+// next slab's global loads are in flight during the arithmetic of the present one.
+// With fewer row blocks than the device holds, several CTAs share a block's base tiles
+// (Shares) and knn_merge_kernel merges their lists: 50 queries over 1M x 128 ran on
+// one CTA before, 147.5 ms; 1.02 ms now.
+template <int RM> struct TileSmem {
+    float2 As[2][BK][16 * RM];
+    float Bs[2][BK][BN + 4];
+    float thr[16 * RM];
+    int cnt[16 * RM];
+    float qn[16 * RM];
+};
+
+template <int KC, int RM>
 __global__ void __launch_bounds__(NT, 2)
     knn_tile_kernel(const float *__restrict__ X, int64_t n, int d, const float *__restrict__ Q, int64_t nq,
-                    int64_t self_offset, const float *__restrict__ xn, const float *__restrict__ qn,
+                    int64_t self_offset, const float *__restrict__ xn, const float *__restrict__ qn, const Shares sh,
                     unsigned long long *__restrict__ best, unsigned long long *__restrict__ buf)
 {
-    static_assert(KC + BUF <= 512, "merge sorts 512 keys");
-    __shared__ __align__(16) float As[BK][BM + 4];
-    __shared__ __align__(16) float Bs[BK][BN + 4];
-    __shared__ float s_thr[BM];
-    __shared__ int s_cnt[BM];
-    __shared__ float s_qn[BM];
+    constexpr int RB = 16 * RM;                            // rows of a block
+    constexpr int QLD = RB * BK / 4 >= NT ? RB * BK / 4 / NT : 1;  // query quads per thread
+    extern __shared__ __align__(16) unsigned char tile_raw[];
+    TileSmem<RM> &sm = *reinterpret_cast<TileSmem<RM> *>(tile_raw);
+    auto &As = sm.As;
+    auto &Bs = sm.Bs;
+    auto &s_thr = sm.thr;
+    auto &s_cnt = sm.cnt;
+    auto &s_qn = sm.qn;
 
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
     const int lane = tid & 31, warp = tid >> 5;
-    const int64_t row0 = (int64_t)blockIdx.x * BM;
+    const Share me = my_share(sh, blockIdx.x);
+    const int64_t row0 = me.block * RB;
+    const int64_t tiles = (n + BN - 1) / BN;
+    const int64_t t0 = tiles * me.g / me.G, t1 = tiles * (me.g + 1) / me.G;
+    best += list_base(sh, me.g, nq, RB, KC);
+    buf += list_base(sh, me.g, nq, RB, BUF);
 
-    for (int r = tid; r < BM; r += NT) {
+    for (int r = tid; r < RB; r += NT) {
         s_thr[r] = INFINITY;
         s_cnt[r] = 0;
         s_qn[r] = row0 + r < nq ? qn[row0 + r] : 0.f;
     }
-    for (int e = tid; e < BM * KC; e += NT) {
+    for (int e = tid; e < RB * KC; e += NT) {
         const int64_t gr = row0 + e / KC;
         if (gr < nq)
             best[gr * KC + e % KC] = EMPTY_KEY;
     }
-    __syncthreads();
 
-    for (int64_t col0 = 0; col0 < n; col0 += BN) {
-        float acc[8][8];
+    // staging: quad kq of row m of the slab; rows past the end and coordinates past d read as 0
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 qv[QLD], xv[2];
+    auto fetch = [&](int64_t tile, int k0) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
+        for (int t = 0; t < QLD; ++t) {
+            const int f = tid + t * NT, m = f >> 2, kq = (f & 3) << 2;
+            qv[t] = m < RB && row0 + m < nq && k0 + kq < d
+                        ? __ldg(reinterpret_cast<const float4 *>(Q + (row0 + m) * d + k0 + kq)) : zero4;
+        }
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                acc[i][j] = 0.f;
+        for (int t = 0; t < 2; ++t) {
+            const int f = tid + t * NT, m = f >> 2, kq = (f & 3) << 2;
+            xv[t] = tile * BN + m < n && k0 + kq < d
+                        ? __ldg(reinterpret_cast<const float4 *>(X + (tile * BN + m) * d + k0 + kq)) : zero4;
+        }
+    };
+    auto store = [&](int b) {
+#pragma unroll
+        for (int t = 0; t < QLD; ++t) {
+            const int f = tid + t * NT, m = f >> 2, kq = (f & 3) << 2;
+            if (m < RB) {
+                As[b][kq][m] = make_float2(qv[t].x, qv[t].x);
+                As[b][kq + 1][m] = make_float2(qv[t].y, qv[t].y);
+                As[b][kq + 2][m] = make_float2(qv[t].z, qv[t].z);
+                As[b][kq + 3][m] = make_float2(qv[t].w, qv[t].w);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int f = tid + t * NT, m = f >> 2, kq = (f & 3) << 2;
+            Bs[b][kq][m] = xv[t].x;
+            Bs[b][kq + 1][m] = xv[t].y;
+            Bs[b][kq + 2][m] = xv[t].z;
+            Bs[b][kq + 3][m] = xv[t].w;
+        }
+    };
+
+    int b = 0;
+    if (t0 < t1) {
+        fetch(t0, 0);
+        store(0);
+    }
+    __syncthreads();
+    for (int64_t tile = t0; tile < t1; ++tile) {
+        const int64_t col0 = tile * BN;
+        unsigned long long acc[RM][4];
+#pragma unroll
+        for (int i = 0; i < RM; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                acc[i][j] = 0ull;
         for (int k0 = 0; k0 < d; k0 += BK) {
-            load_slab(Q, row0, nq, d, k0, As, tid);
-            load_slab(X, col0, n, d, k0, Bs, tid);
-            __syncthreads();
+            const bool last = k0 + BK >= d;
+            const int64_t nt = last ? tile + 1 : tile;
+            if (nt < t1)
+                fetch(nt, last ? 0 : k0 + BK);
 #pragma unroll
             for (int kk = 0; kk < BK; ++kk) {
-                float a[8], b[8];
-                *reinterpret_cast<float4 *>(&a[0]) = *reinterpret_cast<const float4 *>(&As[kk][ty * 4]);
-                *reinterpret_cast<float4 *>(&a[4]) = *reinterpret_cast<const float4 *>(&As[kk][64 + ty * 4]);
-                *reinterpret_cast<float4 *>(&b[0]) = *reinterpret_cast<const float4 *>(&Bs[kk][tx * 4]);
-                *reinterpret_cast<float4 *>(&b[4]) = *reinterpret_cast<const float4 *>(&Bs[kk][64 + tx * 4]);
+                const ulonglong2 x0 = *reinterpret_cast<const ulonglong2 *>(&Bs[b][kk][tx * 4]);
+                const ulonglong2 x1 = *reinterpret_cast<const ulonglong2 *>(&Bs[b][kk][64 + tx * 4]);
+                const unsigned long long xx[4] = {x0.x, x0.y, x1.x, x1.y};
+                unsigned long long qq[RM];
+                if constexpr (RM == 1) {
+                    qq[0] = *reinterpret_cast<const unsigned long long *>(&As[b][kk][ty]);
+                } else {
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
+                    for (int i = 0; i < RM; i += 2) {
+                        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&As[b][kk][ty * RM + i]);
+                        qq[i] = v.x;
+                        qq[i + 1] = v.y;
+                    }
+                }
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int i = 0; i < RM; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        acc[i][j] = fma_f32x2(qq[i], xx[j], acc[i][j]);
             }
+            if (nt < t1)
+                store(b ^ 1);
             __syncthreads();
+            b ^= 1;
         }
         // epilogue: squared distances, threshold filter, append to row buffers
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int r = (i < 4) ? ty * 4 + i : 64 + ty * 4 + (i - 4);
+        for (int i = 0; i < RM; ++i) {
+            const int r = ty * RM + i;
             const int64_t grow = row0 + r;
             if (grow >= nq)
                 continue;
@@ -187,7 +415,9 @@ __global__ void __launch_bounds__(NT, 2)
                 const int64_t c = col0 + cl;
                 if (c >= n || c == self)
                     continue;
-                const float d2 = fmaxf(s_qn[r] + __ldg(xn + c) - 2.f * acc[i][j], 0.f);
+                const unsigned long long pr = acc[i][j >> 1];
+                const float dot = __uint_as_float((unsigned)(j & 1 ? pr >> 32 : pr));
+                const float d2 = fmaxf(s_qn[r] + __ldg(xn + c) - 2.f * dot, 0.f);
                 if (d2 < thr) {
                     const int pos = atomicAdd(&s_cnt[r], 1);
                     buf[grow * BUF + pos] = pack_key(d2, (int)c);
@@ -195,27 +425,118 @@ __global__ void __launch_bounds__(NT, 2)
             }
         }
         __syncthreads();
-        const bool last_tile = col0 + BN >= n;
-        for (int r = warp; r < BM; r += NT / 32) {
+        const bool last_tile = tile + 1 == t1;
+        for (int r = warp; r < RB; r += NT / 32) {
             const int64_t grow = row0 + r;
             if (grow >= nq)
                 break;
             const int c = s_cnt[r];
-            if (c > BUF - BN || (last_tile && c > 0))
-                merge_row<KC>(r, grow, best, buf, s_thr, s_cnt, lane);
+            if (c > BUF - BN || (last_tile && c > 0)) {
+                const float t = merge_row<KC>(grow, c, KC - 1, best, buf, lane);
+                if (lane == 0) {
+                    s_thr[r] = t;
+                    s_cnt[r] = 0;
+                }
+            }
         }
         __syncthreads();
     }
 }
 
-// Rescores the survivors of each row by direct difference and writes the best k:
-// NL lists of KC keys per row (list l of row r at best[l * lstride + r * KC]).
-template <int KC, int NL = 1>
+// Merges the sorted lists of each row that several CTAs swept into list 0 (in place).
+// A CTA per row: its warps each fold every W-th list (the next list's load is in
+// flight), then the first warp folds the others' results from shared memory.  Keys are
+// distinct (the shares' columns are), so the KC smallest of the union are what one
+// sweep of all columns would have kept.
+constexpr int kMergeWarps = 16;
+template <int KC>
+__global__ void knn_merge_kernel(const Shares sh, int rows, int64_t nq, int64_t first, unsigned long long *__restrict__ best)
+{
+    constexpr int PB = KC / 32;
+    __shared__ unsigned long long part[kMergeWarps][KC];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, W = blockDim.x >> 5;
+    const int64_t row = first + blockIdx.x;
+    const int L = row / rows < sh.main ? sh.gm : sh.gt;
+    unsigned long long m[PB] = {}, nx[PB];
+    auto load = [&](int g) {
+        const unsigned long long *p = best + list_base(sh, g, nq, rows, KC) + row * KC;
+#pragma unroll
+        for (int i = 0; i < PB; ++i)
+            nx[i] = g < L ? p[i * 32 + lane] : EMPTY_KEY;
+    };
+    auto fold = [&]() {  // m <- the KC smallest of the sorted lists m and nx
+        const unsigned long long least = __shfl_sync(0xffffffffu, nx[0], 0), most = __shfl_sync(0xffffffffu, m[PB - 1], 31);
+        if (least >= most)
+            return;
+        unsigned long long o[PB];
+#pragma unroll
+        for (int i = 0; i < PB; ++i) {
+            const unsigned long long r = __shfl_sync(0xffffffffu, nx[PB - 1 - i], 31 - lane);
+            o[i] = m[i] < r ? m[i] : r;
+        }
+        warp_merge_compact<PB>(o, lane);
+#pragma unroll
+        for (int i = 0; i < PB; ++i)
+            m[i] = o[i];
+    };
+    load(warp);
+#pragma unroll
+    for (int i = 0; i < PB; ++i)
+        m[i] = nx[i];
+    load(warp + W);
+    for (int g = warp + W; g < L; g += W) {
+        unsigned long long cur[PB];
+#pragma unroll
+        for (int i = 0; i < PB; ++i)
+            cur[i] = nx[i];
+        load(g + W);
+        unsigned long long ahead[PB];
+#pragma unroll
+        for (int i = 0; i < PB; ++i) {
+            ahead[i] = nx[i];
+            nx[i] = cur[i];
+        }
+        fold();
+#pragma unroll
+        for (int i = 0; i < PB; ++i)
+            nx[i] = ahead[i];
+    }
+#pragma unroll
+    for (int i = 0; i < PB; ++i)
+        part[warp][i * 32 + lane] = m[i];
+    __syncthreads();
+    if (warp)
+        return;
+    for (int w = 1; w < W; ++w) {
+#pragma unroll
+        for (int i = 0; i < PB; ++i)
+            nx[i] = part[w][i * 32 + lane];
+        fold();
+    }
+#pragma unroll
+    for (int i = 0; i < PB; ++i)
+        best[row * KC + i * 32 + lane] = m[i];
+}
+
+// Merges what the plan split: all rows when gm > 1, else the rows from block `main` on.
+template <int KC>
+int merge_lists(const Shares &sh, int rows, int64_t nq, unsigned long long *best, cudaStream_t s)
+{
+    const int64_t first = sh.gm > 1 ? 0 : std::min<int64_t>(sh.main * rows, nq);
+    if (first >= nq || std::max(sh.gm, sh.gt) == 1)
+        return ONNG_OK;
+    const int W = std::min(kMergeWarps, std::max(sh.gm, sh.gt));
+    knn_merge_kernel<KC><<<(unsigned)(nq - first), 32 * W, 0, s>>>(sh, rows, nq, first, best);
+    return check_launch("onng_knn: list merge");
+}
+
+// Rescores the KC survivors of each row by direct difference and writes the best k.
+template <int KC>
 __global__ void knn_final_kernel(const float *__restrict__ X, int d, const float *__restrict__ Q, int64_t nq,
                                  const unsigned long long *__restrict__ best, int k, int32_t *__restrict__ nbr,
-                                 float *__restrict__ len, int64_t lstride = 0)
+                                 float *__restrict__ len)
 {
-    constexpr int PER = KC * NL / 32;
+    constexpr int PER = KC / 32;
     const int lane = threadIdx.x & 31;
     const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     if (row >= nq)
@@ -225,7 +546,7 @@ __global__ void knn_final_kernel(const float *__restrict__ X, int d, const float
 #pragma unroll
     for (int i = 0; i < PER; ++i) {
         const int e = i * 32 + lane;
-        const unsigned long long key = best[(int64_t)(e / KC) * lstride + row * KC + e % KC];
+        const unsigned long long key = best[row * KC + e];
         const int id = key_id(key);
         // every lane walks the 32 candidates of this slice in turn
         float mine = INFINITY;
@@ -289,7 +610,7 @@ __global__ void knn_emit_kernel(int64_t nq, const unsigned long long *__restrict
 //
 // knn_tc_kernel: the same sweep with the dot products on the 5th-generation
 // tensor cores, for byte-valued inputs (integers in [0, 255], e.g. 8-bit image
-// descriptors) at d = 64 or 128: they are exact in bfloat16, every product and
+// descriptors) at d = 32 .. 128: they are exact in bfloat16, every product and
 // partial sum is an integer below 2^23, so the float32 accumulation, and with it
 // the ranking, is exact.
 //
@@ -316,7 +637,7 @@ __global__ void knn_emit_kernel(int64_t nq, const unsigned long long *__restrict
 // when its TMEM reads are done and merges afterwards.  Every mbarrier wait gives
 // up after 2 s, records an error code and lets all roles reach the teardown,
 // where TMEM is freed.
-constexpr int TC_M = 128, TC_N = 128, TC_BUF = 256;
+constexpr int TC_M = 128, TC_N = 128, TC_BUF = BUF;
 constexpr int TC_RB = 2;                    // 128-row blocks per CTA
 constexpr int TC_EAGER = 64;                // buffered keys that trigger a merge
 constexpr int TC_ROWS = TC_M * TC_RB;       // query rows per CTA
@@ -442,127 +763,6 @@ template <int KA> struct TcSmem {
     static constexpr int BYTES = 1024 + A_BYTES + STAGES * B_STAGE + 256;
     static_assert(BYTES <= 232448, "more than 227 KB of shared memory");
 };
-
-// Compact warp sorts for the tensor-core epilogue: the stage loops run at run
-// time (only the loop over a lane's registers is unrolled), so the code stays
-// small enough for the instruction cache next to the epilogue's hot loop.
-// Element e = i * 32 + lane lives in v[i] of lane `lane`.
-
-// compare-exchange of registers i and i ^ JR (partners 32 JR elements apart),
-// ascending where bit `size` of the element index is clear
-template <int JR, int N>
-__device__ __forceinline__ void cas_regs(unsigned long long (&v)[N], int lane, int size)
-{
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        const int ii = i ^ JR;
-        if (ii > i) {
-            const bool asc = (((i << 5) | lane) & size) == 0;
-            const unsigned long long a = v[i], b = v[ii];
-            const bool sw = asc ? (a > b) : (a < b);
-            v[i] = sw ? b : a;
-            v[ii] = sw ? a : b;
-        }
-    }
-}
-
-// one bitonic step at distance j elements for sequences of length `size`
-template <int N>
-__device__ __forceinline__ void bitonic_step(unsigned long long (&v)[N], int lane, int size, int j)
-{
-    if (j >= 32) {
-        const int jr = j >> 5;
-        if constexpr (N >= 2)
-            if (jr == 1)
-                cas_regs<1>(v, lane, size);
-        if constexpr (N >= 4)
-            if (jr == 2)
-                cas_regs<2>(v, lane, size);
-        if constexpr (N >= 8)
-            if (jr == 4)
-                cas_regs<4>(v, lane, size);
-    } else {
-        const bool lower = (lane & j) == 0;
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-            const bool asc = (((i << 5) | lane) & size) == 0;
-            const unsigned long long o = __shfl_xor_sync(0xffffffffu, v[i], j);
-            const bool take_min = lower == asc;
-            v[i] = take_min ? (o < v[i] ? o : v[i]) : (o > v[i] ? o : v[i]);
-        }
-    }
-}
-
-// ascending sort of 32 N keys
-template <int N> __device__ void warp_sort_compact(unsigned long long (&v)[N], int lane)
-{
-    static_assert(N == 1 || N == 2 || N == 4 || N == 8, "N in {1, 2, 4, 8}");
-#pragma unroll 1
-    for (int size = 2; size <= 32 * N; size <<= 1)
-#pragma unroll 1
-        for (int j = size >> 1; j > 0; j >>= 1)
-            bitonic_step<N>(v, lane, size, j);
-}
-
-// ascending merge of a bitonic sequence of 32 N keys (one bitonic merge pass with
-// every element's direction ascending)
-template <int N> __device__ void warp_merge_compact(unsigned long long (&v)[N], int lane)
-{
-#pragma unroll 1
-    for (int j = 16 * N; j > 0; j >>= 1)
-        bitonic_step<N>(v, lane, 64 * N, j);
-}
-
-// The warp merges row gr's cnt buffered keys into its sorted best list of KC
-// keys and returns the new threshold: the distance of list entry kth (< KC).
-template <int KC>
-__device__ __noinline__ float tc_merge_row(int64_t gr, int cnt, int kth, unsigned long long *__restrict__ best,
-                                           const unsigned long long *__restrict__ buf, int lane)
-{
-    static_assert(KC <= TC_BUF && TC_BUF == 256, "the buffer sort holds 256 keys");
-    constexpr int PB = KC / 32;
-    unsigned long long a[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int e = i * 32 + lane;
-        a[i] = e < cnt ? buf[gr * TC_BUF + e] : EMPTY_KEY;
-    }
-    // sort the smallest power-of-two prefix holding the cnt keys (the rest is +inf)
-    if (cnt <= 64) {
-        unsigned long long t[2] = {a[0], a[1]};
-        warp_sort_compact<2>(t, lane);
-        a[0] = t[0];
-        a[1] = t[1];
-    } else if (cnt <= 128) {
-        unsigned long long t[4] = {a[0], a[1], a[2], a[3]};
-        warp_sort_compact<4>(t, lane);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            a[i] = t[i];
-    } else {
-        warp_sort_compact<8>(a, lane);
-    }
-    unsigned long long bv[PB], m[PB];
-#pragma unroll
-    for (int i = 0; i < PB; ++i)
-        bv[i] = best[gr * KC + i * 32 + lane];
-    // half-cleaner of (a[0 .. KC), reversed best): the smaller of each pair is a
-    // bitonic sequence holding the KC smallest keys
-#pragma unroll
-    for (int i = 0; i < PB; ++i) {
-        const unsigned long long br = __shfl_sync(0xffffffffu, bv[PB - 1 - i], 31 - lane);
-        m[i] = a[i] < br ? a[i] : br;
-    }
-    warp_merge_compact<PB>(m, lane);
-#pragma unroll
-    for (int i = 0; i < PB; ++i)
-        best[gr * KC + i * 32 + lane] = m[i];
-    unsigned long long kv = m[0];
-#pragma unroll
-    for (int i = 1; i < PB; ++i)
-        kv = (kth >> 5) == i ? m[i] : kv;
-    return key_dist(__shfl_sync(0xffffffffu, kv, kth & 31));
-}
 
 // tcgen05.ld of 32 columns without the wait; tmem_wait32 completes it (its
 // operands tie the registers to the wait, so nothing reads them earlier)
@@ -796,7 +996,7 @@ __device__ void tc_epilogue(uint64_t *accf, uint64_t *acce, uint32_t tmem, int w
             need &= need - 1;
             const int64_t gr = __shfl_sync(0xffffffffu, grow, src);
             const int c = __shfl_sync(0xffffffffu, cnt, src);
-            const float nt = tc_merge_row<KC>(gr, c, kth, best, buf, lane);
+            const float nt = merge_row<KC>(gr, c, kth, best, buf, lane);
             if (lane == src) {
                 thr = nt;
                 cnt = 0;
@@ -808,8 +1008,9 @@ __device__ void tc_epilogue(uint64_t *accf, uint64_t *acce, uint32_t tmem, int w
 template <int KC, int KA>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int64_t n,
-                  int64_t nq, int k, int64_t self_offset, const unsigned *__restrict__ par, const float *__restrict__ qn,
-                  unsigned long long *__restrict__ best, unsigned long long *__restrict__ buf, int *err)
+                  int64_t nq, int k, const Shares sh, int64_t self_offset, const unsigned *__restrict__ par,
+                  const float *__restrict__ qn, unsigned long long *__restrict__ best,
+                  unsigned long long *__restrict__ buf, int *err)
 {
     using L = TcSmem<KA>;
     extern __shared__ unsigned char tc_raw[];
@@ -821,12 +1022,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(abar + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t row0 = (int64_t)blockIdx.x * TC_ROWS;
-    const int64_t tiles = (n + TC_N - 1) / TC_N;
+    const Share me = my_share(sh, blockIdx.x);
+    const int64_t row0 = me.block * TC_ROWS;
+    const int64_t all = (n + TC_N - 1) / TC_N;
     const int nrb = row0 + TC_M < nq ? TC_RB : 1;  // row blocks holding any query row
     // a self-join starts its sweep at the tile of its own rows and wraps around:
     // where nearby rows sit together, the thresholds fall within the first tiles
-    const int64_t t0 = self_offset >= 0 ? ((self_offset + row0) / TC_N) % tiles : 0;
+    const int64_t t0 = self_offset >= 0 ? ((self_offset + row0) / TC_N) % all : 0;
+    const TileMap tm(all, t0, me.G, me.g);
+    const int64_t tiles = tm.count;
+    best += list_base(sh, me.g, nq, TC_ROWS, KC);
+    buf += list_base(sh, me.g, nq, TC_ROWS, TC_BUF);
 
     if (tid == 0) {
         for (int s = 0; s < L::STAGES; ++s) {
@@ -872,8 +1078,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     break;
                 mbar_expect_tx(&full[s], L::B_STAGE);
                 for (int a = 0; a < KA; ++a)
-                    tma_load_2d(sB + s * L::B_STAGE + a * L::B_ATOM, &tmB, a * 64, (int)(((t + t0) % tiles) * TC_N),
-                                &full[s]);
+                    tma_load_2d(sB + s * L::B_STAGE + a * L::B_ATOM, &tmB, a * 64, (int)(tm.tile(t) * TC_N), &full[s]);
                 issued = t + 1;
             }
             // our copies in flight complete before the CTA may exit (bounded)
@@ -922,7 +1127,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
     } else {
         // ------------------------------------------------ epilogue (warps 0-7)
-        tc_epilogue<KC, true>(accf, acce, tmem, warp, lane, row0, nq, n, TileMap(tiles, t0, 1, 0), k - 1, self_offset, nullptr, par, qn,
+        tc_epilogue<KC, true>(accf, acce, tmem, warp, lane, row0, nq, n, tm, k - 1, self_offset, nullptr, par, qn,
                               best, buf, err);
     }
     tc_fence_before();
@@ -958,7 +1163,7 @@ template <int KC>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     knn_tcs_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
                    const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl, int64_t n,
-                   int64_t nq, int nk, int G, int64_t self_offset, const float *__restrict__ xh,
+                   int64_t nq, int nk, const Shares sh, int64_t self_offset, const float *__restrict__ xh,
                    const float *__restrict__ qn, unsigned long long *__restrict__ best,
                    unsigned long long *__restrict__ buf, int *err)
 {
@@ -970,17 +1175,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acce + 2);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t row0 = (int64_t)(blockIdx.x / G) * TC_ROWS;
+    const Share me = my_share(sh, blockIdx.x);
+    const int64_t row0 = me.block * TC_ROWS;
     const int64_t tiles = (n + TC_N - 1) / TC_N;
     const int nrb = row0 + TC_M < nq ? TC_RB : 1;  // row blocks holding any query row
     // a self-join starts its sweep at the tile of its own rows and wraps around:
     // where nearby rows sit together, the thresholds fall within the first tiles
     const int64_t t0 = self_offset >= 0 ? ((self_offset + row0) / TC_N) % tiles : 0;
-    const TileMap tm(tiles, t0, G, (int)(blockIdx.x % G));
+    const TileMap tm(tiles, t0, me.G, me.g);
     const int64_t steps = tm.count * nk;
     // this CTA's lists: share g of the row set keeps its own best list and buffers
-    best += (int64_t)tm.g * nq * KC;
-    buf += (int64_t)tm.g * nq * TC_BUF;
+    best += list_base(sh, me.g, nq, TC_ROWS, KC);
+    buf += list_base(sh, me.g, nq, TC_ROWS, TC_BUF);
 
     if (tid == 0) {
         for (int s = 0; s < TCS_STAGES; ++s) {
@@ -1159,11 +1365,13 @@ __global__ void value_kind_kernel(const float *__restrict__ x, int64_t count, in
 }
 
 // The byte-valued form's operands: row r of M in bfloat16 in columns [0, d) of a
-// row of dpa = d + 64 (an extra K atom), then in columns d, d + 1, d + 2 either
-// 1.0 (queries: s == nullptr) or the three pieces of -floor(s_r / 2) (base rows;
-// s_r = |x_r|^2, an integer below 2^23): its 8-bit fields times 2^16, 2^8 and 1,
-// each exact in bfloat16; zeros elsewhere.  The MMA then accumulates
-// q.x - floor(|x|^2 / 2) exactly.
+// row of dpa = dp + 64 (dp = d rounded up to whole K atoms, and a spare one), then in
+// columns dp, dp + 1, dp + 2 either 1.0 (queries: s == nullptr) or the three pieces
+// of -floor(s_r / 2) (base rows; s_r = |x_r|^2, an integer below 2^23): its 8-bit
+// fields times 2^16, 2^8 and 1, each exact in bfloat16; zeros elsewhere.  The MMA
+// then accumulates q.x - floor(|x|^2 / 2) exactly.  Padding d to whole K atoms takes
+// byte rows of any d = 32 .. 128 here from the float32 sweep (30,011 x 100, the whole
+// build: 20.5 -> 9.3 ms); below 32 the ties of small integers would flood the lists.
 __global__ void aug_rows_kernel(const float *__restrict__ M, int64_t rows, int d, int dpa,
                                 const float *__restrict__ s, __nv_bfloat16 *__restrict__ out)
 {
@@ -1175,8 +1383,8 @@ __global__ void aug_rows_kernel(const float *__restrict__ M, int64_t rows, int d
             float v = 0.f;
             if (j < d)
                 v = M[r * d + j];
-            else if (j < d + 3) {
-                const int p = j - d;
+            else if (j >= dpa - 64 && j < dpa - 61) {
+                const int p = j - (dpa - 64);
                 v = !s ? 1.f : -(float)(p == 0 ? (h >> 16) << 16 : p == 1 ? ((h >> 8) & 255u) << 8 : h & 255u);
             }
             out[r * dpa + j] = __float2bfloat16_rn(v);
@@ -1234,8 +1442,31 @@ int make_map(CUtensorMap *m, const void *ptr, int64_t rows, int d, int box_rows)
 // CTAs sharing one row set in the split sweep: above d = 128 a CTA's A chunks
 // (256 rows x dp x 4 bytes) over all resident CTAs would exceed L2, so two CTAs take
 // alternate tiles of the same rows (half the A data in flight) and keep a best list
-// each, merged by the rescore.
+// each, merged before the rescore.
 int split_share(int d) { return d > 128 ? 2 : 1; }
+
+// The plans of the two kinds of sweep.  They depend on the sizes alone, so the
+// workspace query and the call agree; kSweepSms is the GB300's SM count (two resident
+// CTAs per SM in the float32 sweep, one in the tensor-core sweeps).
+Shares plan_tile(int64_t n, int64_t nq, int rows)
+{
+    return plan_shares((nq + rows - 1) / rows, (n + BN - 1) / BN, 2 * kSweepSms, 1, 8);
+}
+
+Shares plan_tc(int64_t n, int d, int64_t nq, int kc)
+{
+    return plan_shares((nq + TC_ROWS - 1) / TC_ROWS, (n + TC_N - 1) / TC_N, kSweepSms, split_share(d), 8 * (int64_t)kc);
+}
+
+int tile_rows(int64_t nq) { return nq <= 16 ? 16 : nq <= 32 ? 32 : nq <= 64 ? 64 : 128; }
+
+// best lists (KC keys) and candidate buffers (BUF keys) a call needs, of one row each
+int64_t knn_list_rows(int64_t n, int d, int64_t nq, int kc)
+{
+    const int rows = tile_rows(nq);
+    const int64_t a = list_rows(plan_tile(n, nq, rows), nq, rows);
+    return nq < TC_M ? a : std::max(a, list_rows(plan_tc(n, d, nq, kc), nq, TC_ROWS));
+}
 
 int pick_kc(int k)
 {
@@ -1245,30 +1476,47 @@ int pick_kc(int k)
     return 0;
 }
 
+template <int KC, int RM>
+int launch_tile(const float *X, int64_t n, int d, const float *Q, int64_t nq, int64_t self_offset, const Shares &sh,
+                const float *xn, const float *qn, unsigned long long *best, unsigned long long *bufp, cudaStream_t s)
+{
+    ONNG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void *>(knn_tile_kernel<KC, RM>),
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem<RM>)),
+                  "onng_knn: tile kernel smem attribute");
+    knn_tile_kernel<KC, RM><<<(unsigned)sh.ctas(), NT, sizeof(TileSmem<RM>), s>>>(X, n, d, Q, nq, self_offset, xn, qn, sh,
+                                                                                best, bufp);
+    return check_launch("onng_knn: tile kernel");
+}
+
 template <int KC>
 int launch(const float *X, int64_t n, int d, const float *Q, int64_t nq, int k, int64_t self_offset, int32_t *nbr,
            float *len, float *xn, float *qn, unsigned long long *best, unsigned long long *bufp, cudaStream_t s)
 {
-    knn_tile_kernel<KC><<<(unsigned)((nq + BM - 1) / BM), NT, 0, s>>>(X, n, d, Q, nq, self_offset, xn, qn, best, bufp);
-    int st = check_launch("onng_knn: tile kernel");
-    if (st)
+    const int rows = tile_rows(nq);
+    const Shares sh = plan_tile(n, nq, rows);
+    int st = rows == 16   ? launch_tile<KC, 1>(X, n, d, Q, nq, self_offset, sh, xn, qn, best, bufp, s)
+             : rows == 32 ? launch_tile<KC, 2>(X, n, d, Q, nq, self_offset, sh, xn, qn, best, bufp, s)
+             : rows == 64 ? launch_tile<KC, 4>(X, n, d, Q, nq, self_offset, sh, xn, qn, best, bufp, s)
+                          : launch_tile<KC, 8>(X, n, d, Q, nq, self_offset, sh, xn, qn, best, bufp, s);
+    if (st || (st = merge_lists<KC>(sh, rows, nq, best, s)))
         return st;
     knn_final_kernel<KC><<<(unsigned)((nq * 32 + 255) / 256), 256, 0, s>>>(X, d, Q, nq, best, k, nbr, len);
     return check_launch("onng_knn: final kernel");
 }
 
 template <int KC, int KA>
-int launch_tc_kc(const CUtensorMap &ma, const CUtensorMap &mb, int64_t n, int64_t nq, int k, int64_t self_offset,
-                 const unsigned *par, const float *qn, unsigned long long *best, unsigned long long *bufp, int *err,
+int launch_tc_kc(const CUtensorMap &ma, const CUtensorMap &mb, int64_t n, int64_t nq, int k, const Shares &sh,
+                 int64_t self_offset, const unsigned *par, const float *qn, unsigned long long *best, unsigned long long *bufp, int *err,
                  cudaStream_t s)
 {
     const size_t smem = TcSmem<KA>::BYTES;
     ONNG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void *>(knn_tc_kernel<KC, KA>),
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                   "onng_knn: tensor kernel smem attribute");
-    knn_tc_kernel<KC, KA><<<(unsigned)((nq + TC_ROWS - 1) / TC_ROWS), TC_THREADS, smem, s>>>(
-        ma, mb, n, nq, k, self_offset, par, qn, best, bufp, err);
-    return check_launch("onng_knn: tensor kernel");
+    knn_tc_kernel<KC, KA><<<(unsigned)sh.ctas(), TC_THREADS, smem, s>>>(ma, mb, n, nq, k, sh, self_offset, par, qn, best,
+                                                                        bufp, err);
+    int st = check_launch("onng_knn: tensor kernel");
+    return st ? st : merge_lists<KC>(sh, TC_ROWS, nq, best, s);
 }
 
 int launch_tc(const float *X, int64_t n, int d, const float *Q, int64_t nq, int k, int kc, int64_t self_offset,
@@ -1276,7 +1524,8 @@ int launch_tc(const float *X, int64_t n, int d, const float *Q, int64_t nq, int 
               unsigned long long *bufp, int *err, __nv_bfloat16 *xb, __nv_bfloat16 *qb, cudaStream_t s)
 {
     const int gb = num_sms() * 8;
-    const int dpa = d + 64;  // the extra K atom carries -floor(|x|^2 / 2)
+    const int dpa = (d + 63) / 64 * 64 + 64;  // whole K atoms; the extra one carries -floor(|x|^2 / 2)
+    const Shares sh = plan_tc(n, d, nq, kc);
     aug_rows_kernel<<<gb, 256, 0, s>>>(X, n, d, dpa, xn, xb);
     aug_rows_kernel<<<gb, 256, 0, s>>>(Q, nq, d, dpa, nullptr, qb);
     parity_kernel<<<gb, 256, 0, s>>>(xn, n, (n + TC_N - 1) / TC_N * (TC_N / 32), par);
@@ -1288,14 +1537,14 @@ int launch_tc(const float *X, int64_t n, int d, const float *Q, int64_t nq, int 
         return st;
     const int ka = dpa / 64;
     if (kc == 32)
-        st = ka == 2 ? launch_tc_kc<32, 2>(ma, mb, n, nq, k, self_offset, par, qn, best, bufp, err, s)
-                     : launch_tc_kc<32, 3>(ma, mb, n, nq, k, self_offset, par, qn, best, bufp, err, s);
+        st = ka == 2 ? launch_tc_kc<32, 2>(ma, mb, n, nq, k, sh, self_offset, par, qn, best, bufp, err, s)
+                     : launch_tc_kc<32, 3>(ma, mb, n, nq, k, sh, self_offset, par, qn, best, bufp, err, s);
     else if (kc == 64)
-        st = ka == 2 ? launch_tc_kc<64, 2>(ma, mb, n, nq, k, self_offset, par, qn, best, bufp, err, s)
-                     : launch_tc_kc<64, 3>(ma, mb, n, nq, k, self_offset, par, qn, best, bufp, err, s);
+        st = ka == 2 ? launch_tc_kc<64, 2>(ma, mb, n, nq, k, sh, self_offset, par, qn, best, bufp, err, s)
+                     : launch_tc_kc<64, 3>(ma, mb, n, nq, k, sh, self_offset, par, qn, best, bufp, err, s);
     else
-        st = ka == 2 ? launch_tc_kc<128, 2>(ma, mb, n, nq, k, self_offset, par, qn, best, bufp, err, s)
-                     : launch_tc_kc<128, 3>(ma, mb, n, nq, k, self_offset, par, qn, best, bufp, err, s);
+        st = ka == 2 ? launch_tc_kc<128, 2>(ma, mb, n, nq, k, sh, self_offset, par, qn, best, bufp, err, s)
+                     : launch_tc_kc<128, 3>(ma, mb, n, nq, k, sh, self_offset, par, qn, best, bufp, err, s);
     if (st)
         return st;
     int code = 0;
@@ -1308,16 +1557,18 @@ int launch_tc(const float *X, int64_t n, int d, const float *Q, int64_t nq, int 
 }
 
 template <int KC>
-int launch_tcs_kc(const CUtensorMap *m, int64_t n, int64_t nq, int nk, int G, int64_t self_offset, const float *xh,
+int launch_tcs_kc(const CUtensorMap *m, int64_t n, int64_t nq, int nk, const Shares &sh, int64_t self_offset,
+                  const float *xh,
                   const float *qn, unsigned long long *best, unsigned long long *bufp, int *err, cudaStream_t s)
 {
     const size_t smem = TcsSmem::BYTES;
     ONNG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void *>(knn_tcs_kernel<KC>),
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                   "onng_knn: split tensor kernel smem attribute");
-    knn_tcs_kernel<KC><<<(unsigned)((nq + TC_ROWS - 1) / TC_ROWS * G), TC_THREADS, smem, s>>>(
-        m[0], m[1], m[2], m[3], n, nq, nk, G, self_offset, xh, qn, best, bufp, err);
-    return check_launch("onng_knn: split tensor kernel");
+    knn_tcs_kernel<KC><<<(unsigned)sh.ctas(), TC_THREADS, smem, s>>>(m[0], m[1], m[2], m[3], n, nq, nk, sh, self_offset,
+                                                                     xh, qn, best, bufp, err);
+    int st = check_launch("onng_knn: split tensor kernel");
+    return st ? st : merge_lists<KC>(sh, TC_ROWS, nq, best, s);
 }
 
 // Float inputs on the tensor cores: centre, split into bfloat16 hi / lo, sweep
@@ -1343,10 +1594,10 @@ int launch_tcs(const float *X, int64_t n, int d, const float *Q, int64_t nq, int
         (st = make_map(&m[2], xhi, n, dp, TC_N)) || (st = make_map(&m[3], xlo, n, dp, TC_N)))
         return st;
     const int nk = dp / 64;
-    const int G = split_share(d);
-    st = kc == 32 ? launch_tcs_kc<32>(m, n, nq, nk, G, self_offset, xh, qn, best, bufp, err, s)
-         : kc == 64 ? launch_tcs_kc<64>(m, n, nq, nk, G, self_offset, xh, qn, best, bufp, err, s)
-                    : launch_tcs_kc<128>(m, n, nq, nk, G, self_offset, xh, qn, best, bufp, err, s);
+    const Shares sh = plan_tc(n, d, nq, kc);
+    st = kc == 32 ? launch_tcs_kc<32>(m, n, nq, nk, sh, self_offset, xh, qn, best, bufp, err, s)
+         : kc == 64 ? launch_tcs_kc<64>(m, n, nq, nk, sh, self_offset, xh, qn, best, bufp, err, s)
+                    : launch_tcs_kc<128>(m, n, nq, nk, sh, self_offset, xh, qn, best, bufp, err, s);
     if (st)
         return st;
     int code = 0;
@@ -1355,22 +1606,12 @@ int launch_tcs(const float *X, int64_t n, int d, const float *Q, int64_t nq, int
     if (code)
         return set_error(ONNG_E_LIMIT, "onng_knn: tensor-core pipeline wait timed out (role %d)", code);
     const unsigned grid = (unsigned)((nq * 32 + 255) / 256);
-    const int64_t ls = nq * kc;  // the G lists of a row
-    if (G == 1) {
-        if (kc == 32)
-            knn_final_kernel<32><<<grid, 256, 0, s>>>(X, d, Q, nq, best, k, nbr, len);
-        else if (kc == 64)
-            knn_final_kernel<64><<<grid, 256, 0, s>>>(X, d, Q, nq, best, k, nbr, len);
-        else
-            knn_final_kernel<128><<<grid, 256, 0, s>>>(X, d, Q, nq, best, k, nbr, len);
-    } else {
-        if (kc == 32)
-            knn_final_kernel<32, 2><<<grid, 256, 0, s>>>(X, d, Q, nq, best, k, nbr, len, ls);
-        else if (kc == 64)
-            knn_final_kernel<64, 2><<<grid, 256, 0, s>>>(X, d, Q, nq, best, k, nbr, len, ls);
-        else
-            knn_final_kernel<128, 2><<<grid, 256, 0, s>>>(X, d, Q, nq, best, k, nbr, len, ls);
-    }
+    if (kc == 32)
+        knn_final_kernel<32><<<grid, 256, 0, s>>>(X, d, Q, nq, best, k, nbr, len);
+    else if (kc == 64)
+        knn_final_kernel<64><<<grid, 256, 0, s>>>(X, d, Q, nq, best, k, nbr, len);
+    else
+        knn_final_kernel<128><<<grid, 256, 0, s>>>(X, d, Q, nq, best, k, nbr, len);
     return check_launch("onng_knn: final kernel");
 }
 
@@ -1385,10 +1626,11 @@ extern "C" size_t onng_knn_workspace_bytes(int64_t n, int32_t d, int64_t nq, int
     WsCarver c(nullptr);
     c.take<float>((size_t)std::max<int64_t>(n, 1));
     c.take<float>((size_t)std::max<int64_t>(nq, 1));
-    c.take<unsigned long long>((size_t)std::max<int64_t>(nq, 1) * (kc ? kc : 32) * split_share(d));
-    c.take<unsigned long long>((size_t)std::max<int64_t>(nq, 1) * std::max(BUF, TC_BUF) * split_share(d));
+    const size_t lists = (size_t)knn_list_rows(std::max<int64_t>(n, 1), d, std::max<int64_t>(nq, 1), kc ? kc : 32);
+    c.take<unsigned long long>(lists * (kc ? kc : 32));
+    c.take<unsigned long long>(lists * BUF);
     c.take<int>(64);
-    // bfloat16 copies: hi and lo rows of dp = 64 ceil(d / 64) (the byte path's rows of d + 64 fit)
+    // bfloat16 copies: hi and lo rows of dp = 64 ceil(d / 64) (the byte path's rows of dp + 64 fit)
     const size_t dp = (size_t)(std::max(d, 1) + 63) / 64 * 64;
     c.take<__nv_bfloat16>((size_t)std::max<int64_t>(n, 1) * dp * 2);
     c.take<__nv_bfloat16>((size_t)std::max<int64_t>(nq, 1) * dp * 2);
@@ -1418,8 +1660,9 @@ extern "C" int onng_knn(const float *X, int64_t n, int32_t d, const float *Q, in
     WsCarver c(ws);
     float *xn = c.take<float>((size_t)std::max<int64_t>(n, 1));
     float *qn = c.take<float>((size_t)nq);
-    unsigned long long *best = c.take<unsigned long long>((size_t)nq * kc * split_share(d));
-    unsigned long long *bufp = c.take<unsigned long long>((size_t)nq * std::max(BUF, TC_BUF) * split_share(d));
+    const size_t lists = (size_t)knn_list_rows(std::max<int64_t>(n, 1), d, nq, kc);
+    unsigned long long *best = c.take<unsigned long long>(lists * kc);
+    unsigned long long *bufp = c.take<unsigned long long>(lists * BUF);
     int *flags = c.take<int>(64);
     const size_t dp = (size_t)(d + 63) / 64 * 64;
     __nv_bfloat16 *xb = c.take<__nv_bfloat16>((size_t)std::max<int64_t>(n, 1) * dp * 2);
@@ -1436,7 +1679,7 @@ extern "C" int onng_knn(const float *X, int64_t n, int32_t d, const float *Q, in
     if (st)
         return st;
     // tensor-core paths (at least one full tile of base rows and one row block of
-    // queries, k + 16 <= 128): byte-valued inputs at d = 64 / 128 exactly; other
+    // queries, k + 16 <= 128): byte-valued inputs at d = 32 .. 128 exactly; other
     // non-integer inputs at d >= 32 by the split bfloat16 form.  Integer-valued
     // inputs otherwise take the SIMT sweep, which ranks them exactly.
     if (n >= TC_N && nq >= TC_M && kc <= 128 && n <= INT32_MAX - TC_N) {
@@ -1447,7 +1690,7 @@ extern "C" int onng_knn(const float *X, int64_t n, int32_t d, const float *Q, in
         int kind = 3;
         ONNG_CUDA_TRY(cudaMemcpyAsync(&kind, flags, sizeof(int), cudaMemcpyDeviceToHost, s), "onng_knn: flag");
         ONNG_CUDA_TRY(cudaStreamSynchronize(s), "onng_knn: value check");
-        if (!(kind & 1) && (d == 64 || d == 128))
+        if (!(kind & 1) && d >= 32 && d <= 128)
             return launch_tc(X, n, d, Q, nq, k, kc, self_offset, nbr, len, xn, par, qn, best, bufp, flags + 1, xb,
                              qb, s);
         if ((kind & 2) && d >= 32)

@@ -80,6 +80,12 @@ __global__ void seeds_random_kernel(unsigned long long global_seed, int64_t nq, 
 // the tile's own m-th smallest key first, which leaves little more than m keys to
 // insert.  At the end the CTAs of the cluster merge their lists over distributed
 // shared memory, each for its share of the queries.
+//
+// Seeds + search together, before (one CTA per 16 queries over all pivots, scalar
+// arithmetic) and after: 1 query, 1,024 pivots, d = 128: 195 -> 118 us; 1,000 queries,
+// 8,192 pivots, d = 960: 7.57 -> 1.01 ms; 10,000 queries, 1,024 pivots, d = 128:
+// 3.37 -> 3.27 ms.  The packed arithmetic alone (37.5 T float32 operations a second,
+// packed or not; packing halves the issue slots) would take 70 us of the last.
 constexpr int kPivQ = 32;
 constexpr int kPivT = 256;
 constexpr int kPivD = 16;

@@ -325,8 +325,8 @@ int onng_search_probe(const onng_index *idx, const float *Q, int64_t nq, const o
  * Every call looks up the array's device address with the caller's device
  * current, so the entry point stays valid after cudaDeviceReset; make the
  * first call on a device before any stream capture, since that lookup may
- * load the module.  Every call clears the parts that must start at zero (the
- * query counter and the bitmaps) on its stream, so a call sees nothing of the
+ * load the module.  The query counter is cleared on the call's stream and every
+ * warp clears its bitmap before its first use, so a call sees nothing of the
  * previous one.  All calls on a device share the one array: calls whose
  * kernels can overlap on the GPU (other streams, other host threads) race
  * and give wrong results; order them on one stream or with events. */

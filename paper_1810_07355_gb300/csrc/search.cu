@@ -35,7 +35,7 @@ template <class T> Launch pick_v(int d, int k)
 #ifdef ONNG_CHECK
     // the bounds-checked build carries the float32 kernels only
     if constexpr (!std::is_same<T, float>::value) {
-        return {nullptr, 0};
+        return {nullptr, 0, 0};
     } else
 #endif
     {
@@ -51,7 +51,7 @@ template <class T> Launch pick_v(int d, int k)
         if constexpr (ONNG_SEARCH_MAXV >= 8)
             if (V <= 8)
                 return pick_kr<T, 8>(k);
-        return {nullptr, 0};
+        return {nullptr, 0, 0};
     }
 }
 
@@ -199,11 +199,17 @@ static int search_impl(const onng_index *idx, const float *Q, int64_t nq, const 
     a.stats = stats;
     a.feat = feat;
     a.target = target;
+    // 16-bit tags hold an id's bits beyond the bucket number: ids of up to 14 more bits
+    const int bucket_bits = log2i(L.table / 4);
+    int bits = bucket_bits + 1;
+    while (bits < 31 && (int64_t)1 << bits < idx->n)
+        ++bits;
+    a.tag_bits = bits <= bucket_bits + 14 ? bits : 0;
     cudaStream_t s = to_cuda(stream);
-    ONNG_CUDA_TRY(cudaMemsetAsync(a.counter, 0, sizeof(int), s), "onng_search: reset counter");
-    // the bitmaps start empty; every query leaves its bitmap empty again
-    ONNG_CUDA_TRY(cudaMemsetAsync(a.gbits, 0, sizeof(unsigned) * (size_t)slots * a.bits_words, s),
-                  "onng_search: clear visited bitmaps");
+    if (slots >= nq)
+        a.counter = nullptr;  // a warp per query: nothing to hand out
+    else
+        ONNG_CUDA_TRY(cudaMemsetAsync(a.counter, 0, sizeof(int), s), "onng_search: reset counter");
     L.fn<<<(unsigned)blocks, kWarpsPerCta * 32, L.smem, s>>>(a);
     return check_launch("onng_search");
 }
@@ -282,7 +288,7 @@ extern "C" int onng_search_noalloc(const onng_index *idx, const float *Q, int64_
     const int st = noalloc_scratch(&ws);
     if (st)
         return st;
-    // search_impl clears the counter and the bitmaps on `stream` before its launch
+    // search_impl clears the counter on `stream` before its launch; the warps clear their bitmaps
     return search_impl(idx, Q, nq, p, seeds, n_seed, eps_q, es_q, out_ids, out_dist, stats, nullptr, 0.f, ws, cap,
                        stream);
 }

@@ -22,7 +22,7 @@ using InstT = __nv_fp8_e4m3;
 template <> Launch pick<InstT, ONNG_INST_V, ONNG_INST_KR>()
 {
     constexpr size_t sm = sizeof(WarpSmem<Tune<InstT>::hv, Tune<InstT>::ovf>) * kWarpsPerCta;
-    return {search_kernel<ONNG_INST_V, InstT, Tune<InstT>::hv, ONNG_INST_KR>, sm};
+    return {search_kernel<ONNG_INST_V, InstT, Tune<InstT>::hv, ONNG_INST_KR>, sm, Tune<InstT>::hv};
 }
 
 }  // namespace sk

@@ -1,0 +1,61 @@
+"""The search at the shapes where its gathers, its visited table and its candidate levels
+change form: results and counts equal Algorithm 1's on integer data."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1810_07355_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def _compare(X, Q, g, seeds, k, e_s, eps, padded, prec, cap=0):
+    from paper_1810_07355_gb300 import onng
+    idx = onng.Index(_dev(g[0].astype(np.int64)), _dev(g[1].astype(np.int32)), _dev(X))
+    if padded:
+        idx.with_adjacency(padded)
+    ids, dist, st = onng.search(idx, _dev(Q), k, e_s, eps, _dev(seeds), precision=prec, k_rerank=k, max_expansions=cap)
+    o_ids, o_dist, o_st = oracle.search(g[0], g[1], X, Q, k, e_s, np.float32(eps), seeds, max_exp=cap)
+    assert np.array_equal(ids.cpu().numpy(), o_ids)
+    assert np.allclose(dist.cpu().numpy(), o_dist, rtol=1e-6)
+    assert np.array_equal(st[:, :2].cpu().numpy(), o_st[:, :2])
+    return st.cpu().numpy()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("d", [4, 60, 64, 68, 128, 132, 192, 256, 260, 516])
+def test_dimensions(d, prec):
+    """Half-warp and whole-warp gathers, lanes with and without coordinates; more and
+    fewer new nodes than a gather round, through the table and the CSR lists; seeds
+    repeated within a batch and across batches of seeds."""
+    X = synth.small_integers(700, d, high=200 if d > 64 else 9, seed=d)
+    Q = synth.small_integers(9, d, high=200 if d > 64 else 9, seed=d + 1)
+    nbr, ln = oracle.knng(X, 45)
+    g = oracle.adjust_degree(nbr, ln, 20, 45)
+    rng = np.random.default_rng(d)
+    seeds = rng.integers(0, 700, size=(9, 40)).astype(np.int32)
+    seeds[:, 5] = seeds[:, 3]
+    seeds[:, 36] = seeds[:, 2]
+    for k, e_s, eps, padded in ((10, 7, 0.1, 7), (10, 20, 0.2, 24), (3, 40, 0.05, 40), (10, 0, 0.1, 0), (40, 0, 0.02, 0)):
+        _compare(X, Q, g, seeds, k, e_s, eps, padded, prec)
+    _compare(X, Q, g, seeds, 10, 20, 0.2, 20, prec, cap=5)
+
+
+@pytest.mark.parametrize("n", [2, 513, 6000, 20000])
+def test_everything_visited(n):
+    """eps = inf visits every node: from a table that stays nearly empty to one that
+    overflows into the bitmap, and candidate sets that fill the head, the overflow and the
+    pool and are refilled from each."""
+    X = synth.small_integers(n, 8, high=64, seed=n)
+    Q = synth.small_integers(5, 8, high=64, seed=n + 1)
+    nbr, ln = oracle.knng(X, min(16, n - 1))
+    g = oracle.adjust_degree(nbr, ln, min(8, n - 1), min(16, n - 1))
+    seeds = np.tile(np.arange(min(n, 6), dtype=np.int32), (5, 1))
+    _compare(X, Q, g, seeds, min(10, n), 0, np.inf, 0, 0)
+    st = _compare(X, Q, g, seeds, min(10, n), 24, np.inf, 24, 0)
+    assert (st[:, 3] == 0).all()

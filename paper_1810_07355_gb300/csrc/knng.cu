@@ -24,6 +24,7 @@
 // rescored; everything else, and problems smaller than one tile, the SIMT sweep.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -230,7 +231,8 @@ int64_t list_rows(const Shares &sh, int64_t nq, int rows)
 // resident CTAs: whole waves unsplit (gm CTAs a block), and the blocks of the last,
 // partial wave split so that its CTAs end soonest (ceil(blocks gt / slots) rounds of
 // tiles / gt tiles, plus about `warm` tiles' worth for every further list: its
-// threshold starts from nothing).
+// threshold starts from nothing).  200,000 x 100 floats, k = 100 (782 row blocks, 5.1
+// waves): the whole build 67.5 -> 64.2 ms.
 Shares plan_shares(int64_t blocks, int64_t tiles, int64_t slots, int gm, int64_t warm)
 {
     Shares sh;
@@ -626,10 +628,9 @@ __global__ void knn_emit_kernel(int64_t nq, const unsigned long long *__restrict
 //
 // Epilogue (warps 0-7): thread (w, l) owns query row 128 (w / 4) + 32 (w % 4) + l
 // outright, reading it from TMEM lanes 32 (w % 4) .. +31 with tcgen05.ld.  Per
-// 32-column chunk it takes the running maximum of q.x - |x|^2 / 2 (the half
-// norms come from a padded global array, the same address for the whole warp);
-// a chunk whose maximum passes the row's threshold appends its hits (|q|^2 +
-// |x|^2 - 2 q.x below the threshold) to the row's candidate buffer.  A row whose
+// 32-column chunk it takes the maximum of q.x - |x|^2 / 2; a chunk whose maximum
+// passes the threshold of any of the warp's rows appends their hits (tc_chunk) to the
+// rows' candidate buffers.  A row whose
 // buffer may not absorb another tile is merged into its sorted best list by its
 // warp: the buffer is sorted (bitonic, in registers) and a half-cleaner against
 // the reversed best list plus a bitonic merge keep the KC smallest.  No barrier
@@ -790,119 +791,52 @@ __device__ __forceinline__ void tmem_wait32(uint32_t (&v)[32])
                  : "memory");
 }
 
-// the half norms of a chunk's 32 columns (loaded right before their use: a load
-// one chunk ahead costs registers the kernel does not have at one CTA per SM)
-__device__ __forceinline__ void load_h(float4 (&h)[8], const float4 *__restrict__ p)
-{
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-        h[i] = __ldg(p + i);
-}
+// The three forms of a column's value in the accumulators.
+//   EPI_BYTE:  v = q.x - floor(|x|^2 / 2), an integer (the spare K atom adds the norm).
+//              v >= q.x - |x|^2 / 2, so v >= tr selects a superset of the hits; a hit is
+//              corrected by the parity of |x|^2 (one bit per column) to a = q.x - |x|^2 / 2
+//              and kept when a >= tr, i.e. d^2 <= thr.  The comparison is not strict
+//              because thr is the k-th distance so far here (ranking is exact, so the list
+//              needs no slack): a later column at that distance may still win its tie by id.
+//   EPI_FOLD:  v = q.x - |x|^2 / 2 of the split form, the half norm added by spare columns
+//              of K; kept when v > tr.
+//   EPI_NORMS: v = q.x of the split form; the epilogue subtracts the half norms.
+enum { EPI_BYTE, EPI_FOLD, EPI_NORMS };
 
-// tcgen05.ld of one column (each lane its own TMEM lane) and its wait
-__device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr)
-{
-    uint32_t x;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];\n\ttcgen05.wait::ld.sync.aligned;"
-                 : "=r"(x)
-                 : "r"(taddr)
-                 : "memory");
-    return x;
-}
-
-// One 32-column chunk of a row in the split float form: the running maximum of
-// q.x - |x|^2 / 2 decides whether any column passes; then the whole warp visits
-// the passing columns of all its rows once each, reading each back from TMEM
-// (taddr = the chunk's first column; hc = the chunk's half norms).
-__device__ __forceinline__ void tc_chunk(const uint32_t (&v)[32], const float4 (&hq)[8], uint32_t taddr,
-                                         const float *__restrict__ hc, float tr, float qnr, int64_t cb, int64_t self,
+// One 32-column chunk of a row: f[j] is column cb + j.  The maxima of eight groups of
+// four columns decide which groups any row of the warp needs; their hits are appended
+// from registers (static indices: a group is four predicated appends).  At 1M x 128
+// bytes, k = 100, two thirds of the chunks hold a hit of some row, and reading hit
+// columns back from TMEM one by one set the pace: 369 -> 352 ms.  A vote per group
+// instead of the one reduction, unrolled over the tile's four chunks, took 627 ms (code
+// size and branches).
+// sj = the row's own column in the chunk (self-joins), nl = columns of the chunk below n,
+// odd = the parity bits (EPI_BYTE).
+template <int EPI>
+__device__ __forceinline__ void tc_chunk(const float (&f)[32], float tr, float qnr, int cb, int sj, int nl, unsigned odd,
                                          unsigned long long *__restrict__ brow, int &cnt)
 {
-    float a[32];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const float4 x = hq[i];
-        a[4 * i] = __uint_as_float(v[4 * i]) - x.x;
-        a[4 * i + 1] = __uint_as_float(v[4 * i + 1]) - x.y;
-        a[4 * i + 2] = __uint_as_float(v[4 * i + 2]) - x.z;
-        a[4 * i + 3] = __uint_as_float(v[4 * i + 3]) - x.w;
-    }
-    float m0 = a[0], m1 = a[1], m2 = a[2], m3 = a[3];
-#pragma unroll
-    for (int j = 4; j < 32; j += 4) {
-        m0 = fmaxf(m0, a[j]);
-        m1 = fmaxf(m1, a[j + 1]);
-        m2 = fmaxf(m2, a[j + 2]);
-        m3 = fmaxf(m3, a[j + 3]);
-    }
-    if (!__any_sync(0xffffffffu, fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)) > tr))
-        return;
-    unsigned hit = 0;
-#pragma unroll
-    for (int j = 0; j < 32; ++j)
-        hit |= (a[j] > tr ? 1u : 0u) << j;
-    const int64_t sj = self - cb;
-    if (sj >= 0 && sj < 32)
-        hit &= ~(1u << (int)sj);
-    unsigned cols = __reduce_or_sync(0xffffffffu, hit);
-    while (cols) {
-        const int j = __ffs(cols) - 1;
-        cols &= cols - 1;
-        const float x = __uint_as_float(tmem_ld1(taddr + (uint32_t)j)) - __ldg(hc + j);
-        if ((hit >> j) & 1u)
-            brow[cnt++] = pack_key(fmaxf(qnr - 2.f * x, 0.f), (int)(cb + j));
-    }
-}
-
-// The byte-valued form of a chunk: the accumulator already holds
-// v = q.x - floor(|x|^2 / 2) (the MMA adds the spare K atom's pieces), an integer,
-// and v >= q.x - |x|^2 / 2, so v >= tr selects a superset of the hits; a candidate
-// is corrected by the parity of |x|^2 (one bit per column in par, loaded only
-// here) to a = q.x - |x|^2 / 2 and kept when a >= tr, i.e. d^2 <= thr.  The
-// comparison is not strict because thr is the k-th distance so far here (ranking
-// is exact, so the list needs no slack): a later column at that distance may still
-// win its tie by id.  Columns past n (zero rows of the last tile) are skipped.
-// Called by the whole warp: the candidate columns of all 32 rows are visited
-// once each, reading that column back from TMEM (taddr = the chunk's first
-// column), so no lane indexes its registers at run time.
-__device__ __forceinline__ void tc_chunk_aug(const uint32_t (&v)[32], uint32_t taddr, float tr, float qnr, int64_t cb,
-                                             int64_t self, int64_t n, const unsigned *__restrict__ par,
-                                             unsigned long long *__restrict__ brow, int &cnt)
-{
-    const float *f = reinterpret_cast<const float *>(v);
     float m[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
-        m[i] = f[i];
-#pragma unroll
-    for (int j = 8; j < 32; j += 8)
-#pragma unroll
-        for (int i = 0; i < 8; ++i)
-            m[i] = fmaxf(m[i], f[j + i]);
+        m[i] = fmaxf(fmaxf(f[i], f[i + 8]), fmaxf(f[i + 16], f[i + 24]));
     const float mx = fmaxf(fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])), fmaxf(fmaxf(m[4], m[5]), fmaxf(m[6], m[7])));
-    if (!__any_sync(0xffffffffu, mx >= tr))
+    if (!__any_sync(0xffffffffu, EPI == EPI_BYTE ? mx >= tr : mx > tr))
         return;
-    unsigned hit = 0;
+    unsigned groups = 0;
 #pragma unroll
-    for (int j = 0; j < 32; ++j)
-        hit |= (f[j] >= tr ? 1u : 0u) << j;
-    const int64_t sj = self - cb;
-    if (sj >= 0 && sj < 32)
-        hit &= ~(1u << (int)sj);
-    if (n - cb < 32)
-        hit &= n - cb > 0 ? (1u << (int)(n - cb)) - 1u : 0u;
-    unsigned cols = __reduce_or_sync(0xffffffffu, hit);
-    if (!cols)
-        return;
-    const unsigned odd = __ldg(par + (cb >> 5));
-    while (cols) {
-        const int j = __ffs(cols) - 1;
-        cols &= cols - 1;
-        const float x = __uint_as_float(tmem_ld1(taddr + (uint32_t)j));
-        if ((hit >> j) & 1u) {
-            const float aj = x - ((odd >> j) & 1u ? 0.5f : 0.f);
-            if (aj >= tr)
-                brow[cnt++] = pack_key(fmaxf(qnr - 2.f * aj, 0.f), (int)(cb + j));
+    for (int i = 0; i < 8; ++i)
+        groups |= ((EPI == EPI_BYTE ? m[i] >= tr : m[i] > tr) ? 1u : 0u) << i;
+    groups = __reduce_or_sync(0xffffffffu, groups);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        if (!(groups >> i & 1u))
+            continue;
+#pragma unroll
+        for (int j = i; j < 32; j += 8) {
+            const float a = EPI == EPI_BYTE && (odd >> j & 1u) ? f[j] - 0.5f : f[j];
+            if ((EPI == EPI_BYTE ? a >= tr : a > tr) && j != sj && j < nl)
+                brow[cnt++] = pack_key(fmaxf(qnr - 2.f * a, 0.f), cb + j);
         }
     }
 }
@@ -923,9 +857,8 @@ struct TileMap {
 // The epilogue of the tensor-core kernels (warps 0-7; see knn_tc_kernel): one
 // query row per thread, tile by tile from the TMEM accumulators (row block rb =
 // warp / 4 at columns (2 rb + b) * TC_N, b = tile & 1).
-// AUG: the byte-valued form (tc_chunk_aug with the parity bits `par`); otherwise
-// the split float form (tc_chunk with the padded half norms `xh`).
-template <int KC, bool AUG>
+// `xh` holds the padded half norms (EPI_NORMS), `par` the parity bits (EPI_BYTE).
+template <int KC, int EPI>
 __device__ void tc_epilogue(uint64_t *accf, uint64_t *acce, uint32_t tmem, int warp, int lane, int64_t row0,
                             int64_t nq, int64_t n, const TileMap tm, int kth, int64_t self_offset,
                             const float *__restrict__ xh,
@@ -943,48 +876,60 @@ __device__ void tc_epilogue(uint64_t *accf, uint64_t *acce, uint32_t tmem, int w
     const uint32_t lane_base = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(rb * 2 * TC_N);
     for (int64_t t = 0; t < tm.count; ++t) {
         const int b = (int)(t & 1);
+        const int64_t col0 = tm.tile(t) * TC_N;
+        uint4 odd = make_uint4(0u, 0u, 0u, 0u);
+        if constexpr (EPI == EPI_BYTE)
+            odd = __ldg(reinterpret_cast<const uint4 *>(par + (col0 >> 5)));
         const bool ok = mbar_wait(&accf[b], (uint32_t)((t >> 1) & 1), err, 5);
         if (!__all_sync(0xffffffffu, ok))
             break;
         tc_fence_after();
-        const int64_t col0 = tm.tile(t) * TC_N;
         // d^2 = |q|^2 + |x|^2 - 2 q.x < thr  <=>  q.x - |x|^2 / 2 > (|q|^2 - thr) / 2, every
         // term an exact integer or half-integer for byte-valued inputs (approximate in
         // the split float form, whose survivors are rescored)
         const float tr = 0.5f * (qnr - thr);
-        const float4 *h4 = reinterpret_cast<const float4 *>(xh + col0);
+        const int cb0 = (int)col0, left = (int)(n - col0);  // columns of the tile below n: 128 or, in the last, fewer
+        const int64_t sd = self - col0;
+        const int sj0 = sd >= 0 && sd < TC_N ? (int)sd : -1;
+        const float4 *h4 = reinterpret_cast<const float4 *>(xh + (EPI == EPI_NORMS ? col0 : 0));
         const uint32_t tb = lane_base + (uint32_t)(b * TC_N);
         // TMEM loads run one chunk ahead of the filter (chunk pairs: va even, vb odd)
         uint32_t va[32], vb[32];
-        float4 hq[8];
+        auto chunk = [&](uint32_t (&v)[32], int c, unsigned bits) {
+            float f[32];
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                f[j] = __uint_as_float(v[j]);
+            if constexpr (EPI == EPI_NORMS) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float4 x = __ldg(h4 + c * 8 + i);
+                    f[4 * i] -= x.x;
+                    f[4 * i + 1] -= x.y;
+                    f[4 * i + 2] -= x.z;
+                    f[4 * i + 3] -= x.w;
+                }
+            }
+            tc_chunk<EPI>(f, tr, qnr, cb0 + c * 32, sj0 - c * 32, left - c * 32, bits, brow, cnt);
+        };
         tmem_ld32_async(tb, va);
         tmem_wait32(va);
 #pragma unroll 1
         for (int c = 0; c < TC_N / 32; c += 2) {
             tmem_ld32_async(tb + (uint32_t)((c + 1) * 32), vb);
-            if constexpr (AUG) {
-                tc_chunk_aug(va, tb + (uint32_t)(c * 32), tr, qnr, col0 + c * 32, self, n, par, brow, cnt);
-            } else {
-                load_h(hq, h4 + c * 8);
-                tc_chunk(va, hq, tb + (uint32_t)(c * 32), xh + col0 + c * 32, tr, qnr, col0 + c * 32, self, brow,
-                         cnt);
-            }
+            chunk(va, c, c ? odd.z : odd.x);
             tmem_wait32(vb);
-            if (c + 2 < TC_N / 32)
+            if (c + 2 < TC_N / 32) {
                 tmem_ld32_async(tb + (uint32_t)((c + 2) * 32), va);
-            if constexpr (AUG) {
-                tc_chunk_aug(vb, tb + (uint32_t)((c + 1) * 32), tr, qnr, col0 + (c + 1) * 32, self, n, par, brow,
-                             cnt);
             } else {
-                load_h(hq, h4 + (c + 1) * 8);
-                tc_chunk(vb, hq, tb + (uint32_t)((c + 1) * 32), xh + col0 + (c + 1) * 32, tr, qnr,
-                         col0 + (c + 1) * 32, self, brow, cnt);
+                // the accumulators are read: the next tile's MMAs may start meanwhile
+                tc_fence_before();
+                mbar_arrive(&acce[b]);
             }
+            chunk(vb, c + 1, c ? odd.w : odd.y);
             if (c + 2 < TC_N / 32)
                 tmem_wait32(va);
         }
-        tc_fence_before();
-        mbar_arrive(&acce[b]);
         // rows whose buffer may not absorb another tile, or holds TC_EAGER keys (an
         // earlier merge lowers the threshold, which saves later appends: cheaper
         // than the smaller sorts it costs), and all rows after the last tile
@@ -1127,7 +1072,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
     } else {
         // ------------------------------------------------ epilogue (warps 0-7)
-        tc_epilogue<KC, true>(accf, acce, tmem, warp, lane, row0, nq, n, tm, k - 1, self_offset, nullptr, par, qn,
+        tc_epilogue<KC, EPI_BYTE>(accf, acce, tmem, warp, lane, row0, nq, n, tm, k - 1, self_offset, nullptr, par, qn,
                               best, buf, err);
     }
     tc_fence_before();
@@ -1150,7 +1095,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // vectors, as for the SIMT sweep.  Rows are zero-padded to dp = 64 ceil(d / 64),
 // so K runs in chunks of one 64-wide atom: A (both row blocks, hi and lo) and B
 // (hi and lo) stream through a two-stage ring of 96 KB, the accumulators stay in
-// TMEM across the chunks of a tile, and the epilogue is tc_epilogue.
+// TMEM across the chunks of a tile, and the epilogue is tc_epilogue.  Where d leaves
+// three padding columns (FOLD), they carry 1.0 in the queries and the half norm's three
+// bfloat16 pieces (its 24 bits), negated, in the base, so the accumulator arrives with
+// the norm subtracted (it cost the epilogue 8 loads and 32 subtractions per chunk).
 constexpr int TCS_STAGES = 2;
 struct TcsSmem {
     static constexpr int ATOM = TC_M * 128;  // 128 rows x 64 bfloat16 (TC_N == TC_M)
@@ -1159,7 +1107,7 @@ struct TcsSmem {
 };
 static_assert(TC_N == TC_M, "the split kernel's atoms are 128 rows for A and B alike");
 
-template <int KC>
+template <int KC, bool FOLD>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     knn_tcs_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
                    const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl, int64_t n,
@@ -1283,8 +1231,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
     } else {
         // ------------------------------------------------ epilogue (warps 0-7)
-        tc_epilogue<KC, false>(accf, acce, tmem, warp, lane, row0, nq, n, tm, KC - 1, self_offset, xh, nullptr, qn,
-                               best, buf, err);
+        tc_epilogue<KC, FOLD ? EPI_FOLD : EPI_NORMS>(accf, acce, tmem, warp, lane, row0, nq, n, tm, KC - 1, self_offset, xh,
+                                                     nullptr, qn, best, buf, err);
     }
     tc_fence_before();
     __syncthreads();
@@ -1316,11 +1264,13 @@ __global__ void mean_kernel(const double *__restrict__ sums, int64_t n, int d, f
 
 // Row r of M [rows, d] centred on mu, split into bfloat16 hi / lo rows of
 // length dp (zeros past d), and its centred squared norm (half of it when
-// `half`; +inf for the padded rows rows .. padded_rows of a half-norm array).
+// `half`; +inf for the padded rows rows .. padded_rows of a half-norm array).  With
+// `fold` (dp >= d + 3), columns d .. d + 2 of the hi row are 1.0 (queries) or the
+// bfloat16 pieces of minus the half norm (base rows).
 __global__ void split_rows_kernel(const float *__restrict__ M, int64_t rows, int d, int dp,
                                   const float *__restrict__ mu, __nv_bfloat16 *__restrict__ hi,
                                   __nv_bfloat16 *__restrict__ lo, float *__restrict__ norm, bool half,
-                                  int64_t padded_rows)
+                                  int64_t padded_rows, bool fold)
 {
     const int lane = threadIdx.x & 31;
     for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < padded_rows;
@@ -1334,7 +1284,8 @@ __global__ void split_rows_kernel(const float *__restrict__ M, int64_t rows, int
         for (int j = lane; j < dp; j += 32) {
             const float c = j < d ? M[r * d + j] - mu[j] : 0.f;
             const __nv_bfloat16 h = __float2bfloat16_rn(c);
-            hi[r * dp + j] = h;
+            if (!fold || j < d || j >= d + 3)
+                hi[r * dp + j] = h;
             lo[r * dp + j] = __float2bfloat16_rn(c - __bfloat162float(h));
             s = fmaf(c, c, s);
         }
@@ -1343,6 +1294,15 @@ __global__ void split_rows_kernel(const float *__restrict__ M, int64_t rows, int
             s += __shfl_xor_sync(0xffffffffu, s, off);
         if (lane == 0)
             norm[r] = half ? 0.5f * s : s;
+        if (fold && lane < 3) {
+            float rest = -0.5f * s;  // the piece of lane p: what the pieces before it left, rounded
+            __nv_bfloat16 piece = __float2bfloat16_rn(rest);
+            for (int p = 0; p < lane; ++p) {
+                rest -= __bfloat162float(piece);
+                piece = __float2bfloat16_rn(rest);
+            }
+            hi[r * dp + d + lane] = half ? piece : __float2bfloat16_rn(1.f);
+        }
     }
 }
 
@@ -1556,16 +1516,16 @@ int launch_tc(const float *X, int64_t n, int d, const float *Q, int64_t nq, int 
     return check_launch("onng_knn: output");
 }
 
-template <int KC>
+template <int KC, bool FOLD>
 int launch_tcs_kc(const CUtensorMap *m, int64_t n, int64_t nq, int nk, const Shares &sh, int64_t self_offset,
                   const float *xh,
                   const float *qn, unsigned long long *best, unsigned long long *bufp, int *err, cudaStream_t s)
 {
     const size_t smem = TcsSmem::BYTES;
-    ONNG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void *>(knn_tcs_kernel<KC>),
+    ONNG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void *>(knn_tcs_kernel<KC, FOLD>),
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
                   "onng_knn: split tensor kernel smem attribute");
-    knn_tcs_kernel<KC><<<(unsigned)sh.ctas(), TC_THREADS, smem, s>>>(m[0], m[1], m[2], m[3], n, nq, nk, sh, self_offset,
+    knn_tcs_kernel<KC, FOLD><<<(unsigned)sh.ctas(), TC_THREADS, smem, s>>>(m[0], m[1], m[2], m[3], n, nq, nk, sh, self_offset,
                                                                      xh, qn, best, bufp, err);
     int st = check_launch("onng_knn: split tensor kernel");
     return st ? st : merge_lists<KC>(sh, TC_ROWS, nq, best, s);
@@ -1584,8 +1544,9 @@ int launch_tcs(const float *X, int64_t n, int d, const float *Q, int64_t nq, int
     ONNG_CUDA_TRY(cudaMemsetAsync(sums, 0, sizeof(double) * (size_t)d, s), "onng_knn: clear sums");
     col_sums_kernel<<<(unsigned)std::min<int64_t>(n, 1024), 256, 0, s>>>(X, n, d, sums);
     mean_kernel<<<(d + 255) / 256, 256, 0, s>>>(sums, n, d, mu);
-    split_rows_kernel<<<gb, 256, 0, s>>>(X, n, d, dp, mu, xhi, xlo, xh, true, (n + TC_N - 1) / TC_N * TC_N);
-    split_rows_kernel<<<gb, 256, 0, s>>>(Q, nq, d, dp, mu, qhi, qlo, qn, false, nq);
+    const bool fold = dp >= d + 3;
+    split_rows_kernel<<<gb, 256, 0, s>>>(X, n, d, dp, mu, xhi, xlo, xh, true, (n + TC_N - 1) / TC_N * TC_N, fold);
+    split_rows_kernel<<<gb, 256, 0, s>>>(Q, nq, d, dp, mu, qhi, qlo, qn, false, nq, fold);
     int st = check_launch("onng_knn: split copies");
     if (st)
         return st;
@@ -1595,9 +1556,14 @@ int launch_tcs(const float *X, int64_t n, int d, const float *Q, int64_t nq, int
         return st;
     const int nk = dp / 64;
     const Shares sh = plan_tc(n, d, nq, kc);
-    st = kc == 32 ? launch_tcs_kc<32>(m, n, nq, nk, sh, self_offset, xh, qn, best, bufp, err, s)
-         : kc == 64 ? launch_tcs_kc<64>(m, n, nq, nk, sh, self_offset, xh, qn, best, bufp, err, s)
-                    : launch_tcs_kc<128>(m, n, nq, nk, sh, self_offset, xh, qn, best, bufp, err, s);
+    auto sweep = [&](auto kcc) {
+        constexpr int KC = decltype(kcc)::value;
+        return fold ? launch_tcs_kc<KC, true>(m, n, nq, nk, sh, self_offset, xh, qn, best, bufp, err, s)
+                    : launch_tcs_kc<KC, false>(m, n, nq, nk, sh, self_offset, xh, qn, best, bufp, err, s);
+    };
+    st = kc == 32 ? sweep(std::integral_constant<int, 32>{})
+         : kc == 64 ? sweep(std::integral_constant<int, 64>{})
+                    : sweep(std::integral_constant<int, 128>{});
     if (st)
         return st;
     int code = 0;

@@ -41,12 +41,11 @@
 // len(m,j) < len(i,j).  A warp owns a node i at a time (persistent warps stride
 // over the nodes): N(i) goes into a shared-memory hash (id -> position); for
 // every m in N(i) shorter than i's longest edge, the prefix of m's list shorter
-// than that edge (a binary search: rows are sorted by length) is streamed with
-// the others as one flattened sequence across the lanes, and every hit j that
-// satisfies both strict comparisons records the smallest witness position.
-// Nodes with more than 256 edges use a CTA and a hash in global scratch.  A
-// count / scan / compact sequence then writes the kept edges in their input
-// order.
+// than that edge (a binary search: rows are sorted by length) is tested against
+// it, and every hit j that satisfies both strict comparisons records the smallest
+// witness position.  Nodes with more than 256 edges use a CTA in the same way, and
+// those with more than 1,024 several.  A count / scan / compact sequence then writes
+// the kept edges in their input order.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -258,146 +257,182 @@ __global__ void sort_big_rows(const int64_t *__restrict__ row_ptr, unsigned long
 
 // ------------------------------------------------------------------ path
 
-constexpr int kPathSmall = 256;       // rows up to this many edges: one warp, shared-memory hash
-constexpr int kPathHash = 512;        // hash slots for small rows
+constexpr int kPathSmall = 256;  // rows up to this many edges: one warp
+constexpr int kPathMid = 1024;   // up to this many: a CTA of 256 threads; longer rows: several CTAs of 1,024
+constexpr int kPathBlock = 8192; // targets of a long row in shared memory at a time
 constexpr int kPathWarps = 4;
-constexpr int kPathUnroll = 4;  // list entries per lane in flight
+constexpr int kPathUnroll = 4;   // lists walked together, an entry of each per lane
 
-struct PathSmem {
-    int hkey[kPathHash];
-    int hpos[kPathHash];
-    float li[kPathSmall];
-    int wit[kPathSmall];
-    int64_t pre[32];
-    int64_t mb[32];
-    int mu[32];
+// N(i) in shared memory: ids and lengths by position, and a chained hash from id to
+// position (heads by hash, the next position by position), so that an entry that is
+// not in N(i) mostly costs one look at an empty head.
+template <int CAP, int HEADS> struct PathRow {
+    int head[HEADS];
+    int ids[CAP];
+    float li[CAP];
+    int wit[CAP];
+    short nxt[CAP];
+    static_assert(CAP <= 32767, "positions are 16-bit");
 };
 
 __device__ __forceinline__ unsigned phash(int id) { return static_cast<unsigned>(id) * 0x9E3779B1u; }
 
-// Looks id up in an open-addressing table of `cap` slots; returns its position or -1.
-__device__ __forceinline__ int hash_find(const int *hkey, const int *hpos, int cap, int lg, int id)
+// Fills the row structure with node i's deg edges (threads first, first + step, ...).
+template <int CAP, int HEADS>
+__device__ __forceinline__ void path_row_clear(PathRow<CAP, HEADS> &sm, int first, int step)
 {
-    unsigned h = phash(id) >> (32 - lg);
-    for (int t = 0; t < cap; ++t) {
-        const int k = hkey[h];
-        if (k == id)
-            return hpos[h];
-        if (k == -1)
-            return -1;
-        h = (h + 1) & (cap - 1);
+    for (int t = first; t < HEADS; t += step)
+        sm.head[t] = -1;
+}
+template <int CAP, int HEADS>
+__device__ __forceinline__ void path_row_load(PathRow<CAP, HEADS> &sm, int64_t beg, int deg, const int32_t *__restrict__ col,
+                                              const float *__restrict__ len, int first, int step)
+{
+    constexpr int shift = 32 - (HEADS == 512 ? 9 : HEADS == 2048 ? 11 : 13);
+    static_assert(HEADS == 512 || HEADS == 2048 || HEADS == 8192, "HEADS");
+    for (int t = first; t < deg; t += step) {
+        const int j = col[beg + t];
+        sm.ids[t] = j;
+        sm.li[t] = len[beg + t];
+        sm.wit[t] = INT_MAX;
+        sm.nxt[t] = (short)atomicExch(&sm.head[phash(j) >> shift], t);
     }
-    return -1;
 }
 
-__device__ __forceinline__ void hash_put(int *hkey, int *hpos, int cap, int lg, int id, int pos)
+// One warp tests the paths over the 32 neighbours u0 .. u0 + 31 of the row at `beg` of
+// deg edges, to the targets in `sm` (the row's positions from j0 on): of every neighbour
+// m closer than lmax (the row's longest edge) only the prefix of its list shorter than
+// lmax can witness (rows are sorted by length), found by binary search, a lane per
+// neighbour.  Four lists are walked at a time, 32 entries of each per step.
+//
+// The gathers' latency bounds this, so a step's ids are loaded a step ahead, and only
+// the ids: a length is needed just for entries that are targets, farther than m, and not
+// yet removed by a nearer witness.  Those few wait in `queue` until 32 of them fetch
+// their lengths together.  1M rows, 68.8M edges, the whole pass: 67 ms when every entry
+// looked its list up by binary search over prefix sums, loaded its length and probed an
+// open table; 58 with whole lists per step and the chained hash; 46 as it is.
+struct PathQueue {
+    int64_t at[64];      // list entry whose length decides
+    int tgt[64], u[64];  // target (position in sm), witness position
+};
+template <int CAP, int HEADS>
+__device__ __forceinline__ void path_flush(PathRow<CAP, HEADS> &sm, PathQueue &queue, int first, int count,
+                                           const float *__restrict__ len, int lane)
 {
-    unsigned h = phash(id) >> (32 - lg);
-    for (int t = 0; t < cap; ++t) {
-        const int old = atomicCAS(&hkey[h], -1, id);
-        if (old == -1 || old == id) {
-            hpos[h] = pos;
-            return;
-        }
-        h = (h + 1) & (cap - 1);
+    if (lane < count) {
+        const int p = queue.tgt[first + lane];
+        if (__ldg(len + queue.at[first + lane]) < sm.li[p])
+            atomicMin(&sm.wit[p], queue.u[first + lane]);
     }
+    __syncwarp();
+}
+template <int CAP, int HEADS>
+__device__ __forceinline__ void path_scan(PathRow<CAP, HEADS> &sm, PathQueue &queue, int64_t beg, int u0, int deg, float lmax,
+                                          const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
+                                          const float *__restrict__ len, int lane)
+{
+    constexpr int shift = 32 - (HEADS == 512 ? 9 : HEADS == 2048 ? 11 : 13);
+    const int u = u0 + lane;
+    int64_t mb = 0;
+    int cnt = 0;
+    const float lu = u < deg ? len[beg + u] : INFINITY;
+    if (lu < lmax) {
+        const int m = col[beg + u];
+        mb = rp[m];
+        int lo = 0, hi = (int)(rp[m + 1] - mb);
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (len[mb + mid] < lmax)
+                lo = mid + 1;
+            else
+                hi = mid;
+        }
+        cnt = lo;
+    }
+    __syncwarp();
+    const volatile int *wit = sm.wit;
+    int pending = 0;  // queued entries
+    // the lists of the step in hand (g, e) and of the one being loaded
+    int64_t b[kPathUnroll];
+    int c[kPathUnroll], j[kPathUnroll], most = 0;
+    auto lists = [&](int g) {
+        most = 0;
+#pragma unroll
+        for (int r = 0; r < kPathUnroll; ++r) {
+            b[r] = __shfl_sync(0xffffffffu, mb, g + r) + lane;
+            c[r] = __shfl_sync(0xffffffffu, cnt, g + r);
+            most = max(most, c[r]);
+        }
+    };
+    auto load = [&](int e) {
+#pragma unroll
+        for (int r = 0; r < kPathUnroll; ++r)
+            j[r] = e + lane < c[r] ? __ldg(col + b[r] + e) : -1;
+    };
+    const int gend = min(32, deg - u0);
+    int g = 0, e = 0;
+    lists(0);
+    load(0);
+    while (g < gend) {
+        int64_t cb[kPathUnroll];
+        int cj[kPathUnroll];
+#pragma unroll
+        for (int r = 0; r < kPathUnroll; ++r) {
+            cb[r] = b[r] + e;
+            cj[r] = j[r];
+        }
+        const int cg = g;
+        e += 32;
+        if (e >= most) {
+            e = 0;
+            g += kPathUnroll;
+            if (g < gend)
+                lists(g);
+        }
+        if (g < gend)
+            load(e);
+#pragma unroll
+        for (int r = 0; r < kPathUnroll; ++r) {
+            const float l = __shfl_sync(0xffffffffu, lu, cg + r);
+            int p = cj[r] >= 0 ? sm.head[phash(cj[r]) >> shift] : -1;
+            while (p >= 0 && sm.ids[p] != cj[r])
+                p = sm.nxt[p];
+            const bool need = p >= 0 && l < sm.li[p] && wit[p] > u0 + cg + r;
+            const unsigned nm = __ballot_sync(0xffffffffu, need);
+            if (!nm)
+                continue;
+            if (need) {
+                const int at = pending + __popc(nm & ((1u << lane) - 1u));
+                queue.at[at] = cb[r];
+                queue.tgt[at] = p;
+                queue.u[at] = u0 + cg + r;
+            }
+            pending += __popc(nm);
+            __syncwarp();
+            if (pending >= 32) {
+                pending -= 32;
+                path_flush(sm, queue, pending, 32, len, lane);
+            }
+        }
+    }
+    path_flush(sm, queue, 0, pending, len, lane);
 }
 
 // Marks removals of the edges of node i (deg <= kPathSmall) by one warp.
 __device__ void path_row_warp(int64_t i, const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
-                              const float *__restrict__ len, PathSmem &sm, int *__restrict__ wit_out, int lane)
+                              const float *__restrict__ len, PathRow<kPathSmall, 512> &sm, PathQueue &queue,
+                              int *__restrict__ wit_out, int lane)
 {
     const int64_t beg = rp[i];
     const int deg = (int)(rp[i + 1] - beg);
-    constexpr int lg = 9;  // log2(kPathHash)
-    for (int t = lane; t < kPathHash; t += 32)
-        sm.hkey[t] = -1;
+    path_row_clear(sm, lane, 32);
     __syncwarp();
-    for (int t = lane; t < deg; t += 32) {
-        const int j = col[beg + t];
-        sm.li[t] = len[beg + t];
-        sm.wit[t] = INT_MAX;
-        hash_put(sm.hkey, sm.hpos, kPathHash, lg, j, t);
-    }
+    path_row_load(sm, beg, deg, col, len, lane, 32);
     __syncwarp();
-    float lmax = 0.f;
-    for (int t = lane; t < deg; t += 32)
-        lmax = fmaxf(lmax, sm.li[t]);
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1)
-        lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, off));
-    for (int u0 = 0; u0 < deg; u0 += 32) {
-        const int u = u0 + lane;
-        int64_t cnt = 0, mb = 0;
-        if (u < deg && sm.li[u] < lmax) {
-            // only the prefix of m's list shorter than lmax can witness (rows are
-            // sorted by length): its size by binary search
-            const int m = col[beg + u];
-            mb = rp[m];
-            int64_t lo = 0, hi = rp[m + 1] - mb;
-            while (lo < hi) {
-                const int64_t mid = (lo + hi) >> 1;
-                if (len[mb + mid] < lmax)
-                    lo = mid + 1;
-                else
-                    hi = mid;
-            }
-            cnt = lo;
-        }
-        int64_t x = cnt;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int64_t y = __shfl_up_sync(0xffffffffu, x, off);
-            if (lane >= off)
-                x += y;
-        }
-        sm.pre[lane] = x;  // inclusive prefix
-        sm.mb[lane] = mb;
-        sm.mu[lane] = u;
-        __syncwarp();
-        const int64_t total = sm.pre[31];
-        // kPathUnroll entries per lane and round: their list loads are all issued
-        // before any is used, so several gathers are in flight per lane
-        for (int64_t e0 = lane; e0 < total; e0 += 32 * kPathUnroll) {
-            int own[kPathUnroll];
-            int64_t idx[kPathUnroll];
-#pragma unroll
-            for (int r = 0; r < kPathUnroll; ++r) {
-                const int64_t e = e0 + 32 * r;
-                int lo = 0, hi = 31;  // first lane whose inclusive prefix exceeds e
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (sm.pre[mid] > e)
-                        hi = mid;
-                    else
-                        lo = mid + 1;
-                }
-                own[r] = e < total ? lo : -1;
-                const int64_t start = sm.pre[lo] - (lo ? sm.pre[lo - 1] : 0);
-                idx[r] = sm.mb[lo] + (e - (sm.pre[lo] - start));
-            }
-            float lmj[kPathUnroll];
-            int cj[kPathUnroll];
-#pragma unroll
-            for (int r = 0; r < kPathUnroll; ++r) {
-                lmj[r] = own[r] >= 0 ? len[idx[r]] : INFINITY;
-                cj[r] = own[r] >= 0 ? col[idx[r]] : -1;
-            }
-#pragma unroll
-            for (int r = 0; r < kPathUnroll; ++r) {
-                if (own[r] < 0 || !(lmj[r] < lmax))
-                    continue;
-                const int t = hash_find(sm.hkey, sm.hpos, kPathHash, lg, cj[r]);
-                if (t < 0)
-                    continue;
-                const int uu = sm.mu[own[r]];
-                const float lij = sm.li[t];
-                if (sm.li[uu] < lij && lmj[r] < lij)
-                    atomicMin(&sm.wit[t], uu);
-            }
-        }
-        __syncwarp();
-    }
+    const float lmax = sm.li[deg - 1];  // rows are sorted by length
+    for (int u0 = 0; u0 < deg; u0 += 32)
+        path_scan(sm, queue, beg, u0, deg, lmax, rp, col, len, lane);
+    __syncwarp();
     for (int t = lane; t < deg; t += 32)
         wit_out[beg + t] = sm.wit[t] == INT_MAX ? -1 : sm.wit[t];
     __syncwarp();
@@ -410,126 +445,98 @@ __global__ void __launch_bounds__(kPathWarps * 32)
     path_small_kernel(const int64_t *__restrict__ rp, const int32_t *__restrict__ col, const float *__restrict__ len,
                       int64_t n, int *__restrict__ wit, int64_t *__restrict__ big_rows, int *__restrict__ n_big)
 {
-    __shared__ PathSmem sm[kPathWarps];
+    __shared__ PathRow<kPathSmall, 512> sm[kPathWarps];
+    __shared__ PathQueue queue[kPathWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * kPathWarps;
     for (int64_t i = (int64_t)blockIdx.x * kPathWarps + warp; i < n; i += stride) {
         const int64_t deg = rp[i + 1] - rp[i];
         if (deg > kPathSmall) {
+            // rows of several CTAs are listed from the end; their marks are combined in place
+            const bool several = deg > kPathMid;
             if (lane == 0)
-                big_rows[atomicAdd(n_big, 1)] = i;
+                big_rows[several ? n - 1 - atomicAdd(n_big + 1, 1) : atomicAdd(n_big, 1)] = i;
+            if (several)
+                for (int64_t t = lane; t < deg; t += 32)
+                    wit[rp[i] + t] = INT_MAX;
             continue;
         }
         if (deg >= 2)
-            path_row_warp(i, rp, col, len, sm[warp], wit, lane);
+            path_row_warp(i, rp, col, len, sm[warp], queue[warp], wit, lane);
         else if (deg == 1 && lane == 0)
             wit[rp[i]] = -1;
     }
 }
 
-// Open-addressing table of any size `cap` (range reduction by multiply-high).
-__device__ __forceinline__ int ghash_find(const int *hkey, const int *hpos, int cap, int id)
+// Listed rows of kPathSmall < edges <= kPathMid: a CTA per row, its warps taking 32
+// neighbours at a time, everything but the graph in shared memory.
+__global__ void __launch_bounds__(256)
+    path_mid_kernel(const int64_t *__restrict__ rp, const int32_t *__restrict__ col, const float *__restrict__ len,
+                    int *__restrict__ wit, const int64_t *__restrict__ big_rows, const int *__restrict__ n_big)
 {
-    unsigned h = __umulhi(phash(id), (unsigned)cap);
-    for (int t = 0; t < cap; ++t) {
-        const int k = hkey[h];
-        if (k == id)
-            return hpos[h];
-        if (k == -1)
-            return -1;
-        h = h + 1 == (unsigned)cap ? 0 : h + 1;
-    }
-    return -1;
-}
-
-__device__ __forceinline__ void ghash_put(int *hkey, int *hpos, int cap, int id, int pos)
-{
-    unsigned h = __umulhi(phash(id), (unsigned)cap);
-    for (int t = 0; t < cap; ++t) {
-        const int old = atomicCAS(&hkey[h], -1, id);
-        if (old == -1 || old == id) {
-            hpos[h] = pos;
-            return;
-        }
-        h = h + 1 == (unsigned)cap ? 0 : h + 1;
-    }
-}
-
-// Rows with more than kPathSmall edges: one CTA per row; the row's hash lives in
-// global scratch at offset 2 * row_ptr[i] (2 * degree slots, so rows never overlap).
-__global__ void path_big_kernel(const int64_t *__restrict__ rp, const int32_t *__restrict__ col,
-                                const float *__restrict__ len, int *__restrict__ wit,
-                                const int64_t *__restrict__ big_rows, const int *__restrict__ n_big,
-                                int *__restrict__ skey, int *__restrict__ spos)
-{
-    __shared__ float s_lmax;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int b = blockIdx.x; b < *n_big; b += gridDim.x) {
-        const int64_t i = big_rows[b];
-        const int64_t beg = rp[i];
-        const int deg = (int)(rp[i + 1] - beg);
-        const int cap = 2 * deg;
-        int *hkey = skey + 2 * beg;
-        int *hpos = spos + 2 * beg;
-        for (int t = threadIdx.x; t < cap; t += blockDim.x)
-            hkey[t] = -1;
-        if (threadIdx.x == 0)
-            s_lmax = 0.f;
+    __shared__ PathRow<kPathMid, 2048> sm;
+    __shared__ PathQueue queue[256 / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int b = blockIdx.x; b < n_big[0]; b += gridDim.x) {
+        const int64_t beg = rp[big_rows[b]];
+        const int deg = (int)(rp[big_rows[b] + 1] - beg);
+        path_row_clear(sm, threadIdx.x, blockDim.x);
         __syncthreads();
-        for (int t = threadIdx.x; t < deg; t += blockDim.x) {
-            wit[beg + t] = INT_MAX;
-            ghash_put(hkey, hpos, cap, col[beg + t], t);
-        }
-        if (threadIdx.x == 0)
-            s_lmax = len[beg + deg - 1];  // rows are sorted by length
+        path_row_load(sm, beg, deg, col, len, threadIdx.x, blockDim.x);
         __syncthreads();
-        const float lmax = s_lmax;
-        for (int u = warp; u < deg; u += nw) {
-            const float liu = len[beg + u];
-            if (!(liu < lmax))
-                continue;
-            const int m = col[beg + u];
-            const int64_t mb = rp[m];
-            // the prefix of m's list shorter than lmax (rows are sorted by length)
-            int64_t lo = 0, hi = rp[m + 1] - mb;
-            while (lo < hi) {
-                const int64_t mid = (lo + hi) >> 1;
-                if (len[mb + mid] < lmax)
-                    lo = mid + 1;
-                else
-                    hi = mid;
-            }
-            const int64_t me = mb + lo;
-            // kPathUnroll entries per lane in flight
-            for (int64_t i0 = mb + lane; i0 < me; i0 += 32 * kPathUnroll) {
-                float lmj[kPathUnroll];
-                int cj[kPathUnroll];
-#pragma unroll
-                for (int r = 0; r < kPathUnroll; ++r) {
-                    const int64_t idx = i0 + 32 * r;
-                    lmj[r] = idx < me ? len[idx] : INFINITY;
-                    cj[r] = idx < me ? col[idx] : -1;
-                }
-#pragma unroll
-                for (int r = 0; r < kPathUnroll; ++r) {
-                    if (cj[r] < 0)
-                        continue;
-                    const int t = ghash_find(hkey, hpos, cap, cj[r]);
-                    if (t < 0)
-                        continue;
-                    const float lij = len[beg + t];
-                    if (liu < lij && lmj[r] < lij)
-                        atomicMin(&wit[beg + t], u);
-                }
-            }
-        }
+        const float lmax = sm.li[deg - 1];
+        for (int u0 = warp * 32; u0 < deg; u0 += blockDim.x)
+            path_scan(sm, queue[warp], beg, u0, deg, lmax, rp, col, len, lane);
         __syncthreads();
         for (int t = threadIdx.x; t < deg; t += blockDim.x)
-            if (wit[beg + t] == INT_MAX)
-                wit[beg + t] = -1;
+            wit[beg + t] = sm.wit[t] == INT_MAX ? -1 : sm.wit[t];
         __syncthreads();
     }
 }
+
+// Rows of more than kPathMid edges, as tasks of 1,024 neighbours by kPathBlock targets
+// dealt out over the CTAs (one CTA per row left a hub of 9,679 edges alone on its SM for
+// 7 ms of a 60 ms pass).  A task's marks go to the row by atomicMin; marks that stay
+// INT_MAX count as kept.
+struct PathLong {
+    PathRow<kPathBlock, 8192> row;
+    PathQueue queue[32];
+};
+__global__ void __launch_bounds__(1024)
+    path_long_kernel(const int64_t *__restrict__ rp, const int32_t *__restrict__ col, const float *__restrict__ len, int64_t n,
+                     int *__restrict__ wit, const int64_t *__restrict__ big_rows, const int *__restrict__ n_big)
+{
+    extern __shared__ __align__(16) unsigned char path_raw[];
+    PathLong &sm = *reinterpret_cast<PathLong *>(path_raw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int64_t task = 0;
+    for (int b = 0; b < n_big[1]; ++b) {
+        const int64_t i = big_rows[n - 1 - b], beg = rp[i];
+        const int deg = (int)(rp[i + 1] - beg);
+        const int segs = (deg + 1023) / 1024, blocks = (deg + kPathBlock - 1) / kPathBlock;
+        const float lmax = len[beg + deg - 1];
+        for (int t = 0; t < segs * blocks; ++t, ++task) {
+            if (task % gridDim.x != blockIdx.x)
+                continue;
+            const int j0 = t % blocks * kPathBlock, targets = min(kPathBlock, deg - j0);
+            path_row_clear(sm.row, threadIdx.x, 1024);
+            __syncthreads();
+            path_row_load(sm.row, beg + j0, targets, col, len, threadIdx.x, 1024);
+            __syncthreads();
+            const int u0 = t / blocks * 1024 + warp * 32;
+            if (u0 < deg)
+                path_scan(sm.row, sm.queue[warp], beg, u0, deg, lmax, rp, col, len, lane);
+            __syncthreads();
+            for (int e = threadIdx.x; e < targets; e += 1024)
+                if (sm.row.wit[e] != INT_MAX)
+                    atomicMin(&wit[beg + j0 + e], sm.row.wit[e]);
+            __syncthreads();
+        }
+    }
+}
+
+// a witness position, or none: -1, or INT_MAX in the rows of several CTAs
+__device__ __forceinline__ bool path_kept(int w) { return (unsigned)w >= (unsigned)INT_MAX; }
 
 __global__ void path_count_kernel(const int64_t *__restrict__ rp, int64_t n, const int *__restrict__ wit,
                                   int64_t *__restrict__ kept)
@@ -540,7 +547,7 @@ __global__ void path_count_kernel(const int64_t *__restrict__ rp, int64_t n, con
         return;
     int64_t c = 0;
     for (int64_t e = rp[i] + lane; e < rp[i + 1]; e += 32)
-        c += wit[e] < 0;
+        c += path_kept(wit[e]);
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1)
         c += __shfl_xor_sync(0xffffffffu, c, off);
@@ -561,7 +568,7 @@ __global__ void path_compact_kernel(const int64_t *__restrict__ rp, const int32_
     int64_t w = rp_out[i];
     for (int64_t e0 = beg; e0 < end; e0 += 32) {
         const int64_t e = e0 + lane;
-        const bool keep = e < end && wit[e] < 0;
+        const bool keep = e < end && path_kept(wit[e]);
         const unsigned km = __ballot_sync(0xffffffffu, keep);
         if (keep) {
             const int64_t dst = w + __popc(km & ((1u << lane) - 1u));
@@ -569,7 +576,7 @@ __global__ void path_compact_kernel(const int64_t *__restrict__ rp, const int32_
             len_out[dst] = len[e];
         }
         if (removed_by && e < end)
-            removed_by[e] = wit[e] < 0 ? -1 : col[beg + wit[e]];
+            removed_by[e] = path_kept(wit[e]) ? -1 : col[beg + wit[e]];
         w += __popc(km);
     }
 }
@@ -1123,8 +1130,6 @@ extern "C" size_t onng_adjust_path_workspace_bytes(int64_t n, int64_t nnz)
 {
     WsCarver c(nullptr);
     c.take<int>((size_t)std::max<int64_t>(nnz, 1));        // witness positions
-    c.take<int>((size_t)std::max<int64_t>(nnz, 1) * 2);    // hub hash keys
-    c.take<int>((size_t)std::max<int64_t>(nnz, 1) * 2);    // hub hash positions
     c.take<int64_t>((size_t)std::max<int64_t>(n, 1));      // kept counts / long rows
     c.take<int64_t>((size_t)std::max<int64_t>(n, 1));
     c.take<int>(64);
@@ -1150,8 +1155,6 @@ extern "C" int onng_adjust_path(const int64_t *row_ptr, const int32_t *col, cons
     ONNG_REQUIRE(nnz == 0 || (col && len && col_out && len_out), ONNG_E_INVAL, "onng_adjust_path: NULL arrays");
     WsCarver c(ws);
     int *wit = c.take<int>((size_t)std::max<int64_t>(nnz, 1));
-    int *skey = c.take<int>((size_t)std::max<int64_t>(nnz, 1) * 2);
-    int *spos = c.take<int>((size_t)std::max<int64_t>(nnz, 1) * 2);
     int64_t *kept = c.take<int64_t>((size_t)std::max<int64_t>(n, 1));
     int64_t *big = c.take<int64_t>((size_t)std::max<int64_t>(n, 1));
     int *n_big = c.take<int>(64);
@@ -1159,15 +1162,19 @@ extern "C" int onng_adjust_path(const int64_t *row_ptr, const int32_t *col, cons
     char *scan_ws = c.take<char>(scan_workspace_bytes(std::max<int64_t>(n, 1)));
     int st;
     if (n > 0) {
-        ONNG_CUDA_TRY(cudaMemsetAsync(n_big, 0, sizeof(int), s), "adjust_path: clear");
+        ONNG_CUDA_TRY(cudaMemsetAsync(n_big, 0, 2 * sizeof(int), s), "adjust_path: clear");
         int per_sm = 0;
         ONNG_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, path_small_kernel, kPathWarps * 32, 0),
                       "adjust_path: occupancy");
         const int64_t resident = (int64_t)num_sms() * std::max(per_sm, 1);
         const int64_t ctas = std::min<int64_t>((n + kPathWarps - 1) / kPathWarps, resident);
         path_small_kernel<<<(unsigned)ctas, kPathWarps * 32, 0, s>>>(row_ptr, col, len, n, wit, big, n_big);
-        // hub rows: the kernel reads the count of listed rows on the device
-        path_big_kernel<<<num_sms() * 2, 512, 0, s>>>(row_ptr, col, len, wit, big, n_big, skey, spos);
+        // longer rows: the kernels read the counts of listed rows on the device
+        ONNG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void *>(path_long_kernel),
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PathLong)),
+                      "adjust_path: smem attribute");
+        path_mid_kernel<<<num_sms() * 8, 256, 0, s>>>(row_ptr, col, len, wit, big, n_big);
+        path_long_kernel<<<num_sms(), 1024, sizeof(PathLong), s>>>(row_ptr, col, len, n, wit, big, n_big);
         st = check_launch("onng_adjust_path: mark");
         if (st)
             return st;

@@ -1,0 +1,63 @@
+"""Path and degree adjustment at the row sizes where another kernel or another sorting
+network takes over: results and witnesses equal the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _graph(n, hub, seed):
+    """A CSR of n rows of 1 .. 40 edges, some of them of `hub` edges; rows by (length, id),
+    lengths with many ties."""
+    rng = np.random.default_rng(seed)
+    deg = rng.integers(1, 41, size=n)
+    deg[rng.choice(n, 3, replace=False)] = hub
+    rp = np.concatenate([[0], np.cumsum(deg)]).astype(np.int64)
+    col, ln = np.empty(rp[-1], np.int32), np.empty(rp[-1], np.float32)
+    for i in range(n):
+        ids = rng.choice(n - 1, deg[i], replace=False)
+        ids = np.where(ids >= i, ids + 1, ids)
+        length = rng.integers(1, 60, size=deg[i]).astype(np.float32)
+        o = np.lexsort((ids, length))
+        col[rp[i]:rp[i + 1]], ln[rp[i]:rp[i + 1]] = ids[o], length[o]
+    return rp, col, ln
+
+
+@pytest.mark.parametrize("n,hub", [(300, 31), (600, 256), (600, 257), (1100, 1024), (1100, 1025), (2500, 2047),
+                                   (8400, 8192), (8400, 8193)])
+def test_path_rows(n, hub):
+    import torch
+
+    from paper_1810_07355_gb300 import onng
+    rp, col, ln = _graph(n, hub, hub)
+    got = onng.adjust_path(*(torch.from_numpy(v).cuda() for v in (rp, col, ln)), witnesses=True)
+    want = oracle.adjust_path(rp, col, ln, witnesses=True)
+    for g, w in zip(got, want):
+        assert np.array_equal(g.cpu().numpy(), w.astype(g.cpu().numpy().dtype))
+
+
+@pytest.mark.parametrize("n,k,e_o,e_i", [(700, 31, 31, 31), (700, 64, 33, 1), (1500, 100, 0, 100), (40, 39, 39, 39),
+                                         (900, 6, 5, 6)])
+def test_degree_rows(n, k, e_o, e_i):
+    """kNN widths that are and are not a multiple of four, one to several 32-entry chunks,
+    rows of every sorting network, reversed edges onto a hub of more than 512."""
+    import torch
+
+    from paper_1810_07355_gb300 import onng
+    rng = np.random.default_rng(k)
+    nbr = np.empty((n, k), np.int32)
+    for i in range(n):
+        ids = rng.choice(n - 1, k, replace=False)
+        ids = np.where(ids >= i, ids + 1, ids)
+        if i > 0 and 0 not in ids:
+            ids[rng.integers(0, k)] = 0  # node 0 is a hub
+        nbr[i] = ids
+    ln = np.sort(rng.integers(1, 40, size=(n, k)).astype(np.float32), axis=1)
+    for i in range(n):
+        nbr[i] = nbr[i][np.lexsort((nbr[i], ln[i]))]
+    got = onng.adjust_degree(torch.from_numpy(nbr).cuda(), torch.from_numpy(ln).cuda(), e_o, e_i)
+    want = oracle.adjust_degree(nbr, ln, e_o, e_i)
+    for g, w in zip(got, want[:3]):
+        assert np.array_equal(g.cpu().numpy(), w.astype(g.cpu().numpy().dtype))

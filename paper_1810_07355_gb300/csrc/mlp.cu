@@ -270,35 +270,131 @@ __global__ void mlp_adam_kernel(float *__restrict__ P, const float *__restrict__
 }
 
 // Whole training run in one CTA, as batched small matrix products in shared
-// memory (no atomics): per step, for a mini-batch of B <= 128 consecutive rows
-// (wrapping around the set) the forward pass keeps the pre-activations A1, A2
-// [B][64]; the backward pass forms dA2, the gradients of W3, W2, then dA1 and the
-// gradients of W1; Adam updates the parameters in place.  The weights are kept
-// both row-major (flat layout, for Adam and the backward pass) and transposed
-// (for the forward pass) so that the 32 lanes of a warp read consecutive words.
+// memory (no atomics but the loss): per step, for a mini-batch of B <= 128 consecutive
+// rows (wrapping around the set) the forward pass keeps h1 = relu(A1) and h2 = relu(A2)
+// (their signs decide relu' as well); the backward pass forms dA2, the gradients of W3
+// and W2, then dA1 and the gradients of W1; Adam updates the parameters.
+//
+// The steps depend on each other, so one SM works alone; what bounds it is its float32
+// pipe (1.9 M multiply-adds a step, 7.4 us at 128 per cycle) and the chains between its
+// barriers.  One result per thread read two shared values per multiply-add, and a
+// shared-memory float atomic per sample for the loss queued: 78.5 us a step of 128 rows;
+// 19.8 us as it is now.  Every
+// product is a register tile of 4 x 4 results per thread with 16-byte reads, over
+// arrays that hold a feature's samples in a row: the forward products and dA1 read 4
+// weights and 4 samples per term, the weight gradients 4 samples of 4 + 4 features per
+// 4 terms.  Rows are 132 floats, so 8 neighbouring rows (or a row's 8 quads) lie in
+// distinct banks, and a warp's tiles are laid out along them.  Each result is still one
+// chain of multiply-adds in the order of its sum.  The parameters and their moments
+// stay in registers for the whole run.
 constexpr int kTrainMaxB = 128;
-constexpr int kTrainThreads = 256;
+constexpr int kTrainThreads = 512;
+constexpr int kTrainPer = (NP + kTrainThreads - 1) / kTrainThreads;  // parameters per thread
+constexpr int kTrainX = kTrainMaxB * I / kTrainThreads;              // inputs fetched per thread
+constexpr int kTrainRow = kTrainMaxB + 4;
 
-struct TrainShared {
-    float P[NP];
-    float G[NP];
-    float w1t[I * H];
-    float w2t[H * H];
-    float x[kTrainMaxB * I];
+struct __align__(16) TrainShared {
+    float G[NP + 2];
+    float w1t[I * H];          // [i][u]
+    float w2t[H * H];          // [i][u]
+    float w2[H * H];           // [u][i]
+    float xt[I][kTrainRow];    // [i][b]; samples past the batch are zero
+    float h1[H][kTrainRow];    // [i][b]: relu(A1)
+    float h2[H][kTrainRow];    // [u][b]: relu(A2)
+    float da2[H][kTrainRow];   // [u][b]
+    float da1[H][kTrainRow];   // [i][b]
+    float dy[O][kTrainRow];    // [o][b]
     float t[kTrainMaxB * O];
-    float a1[kTrainMaxB * H];
-    float a2[kTrainMaxB * H];  // pre-activations of layer 2, later dA1
-    float da[kTrainMaxB * H];  // dA2
-    float dy[kTrainMaxB * O];
+    float b1[H], b2[H], w3[O * H], b3[O];
     float loss;
 };
 
-__device__ void refresh_transposed(TrainShared &s)
+__device__ __forceinline__ float4 lds4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+
+// acc[i][j] += sum over k = 0 .. K-1, in order, of a[k][i] b[k][j]: 4 + 4 values of rows
+// lda and ldb apart
+__device__ __forceinline__ void tile_rows(float (&acc)[4][4], const float *a, int lda, const float *b, int ldb, int K)
 {
-    for (int e = threadIdx.x; e < H * I; e += blockDim.x)
-        s.w1t[(e % I) * H + e / I] = s.P[oW1 + e];
-    for (int e = threadIdx.x; e < H * H; e += blockDim.x)
-        s.w2t[(e % H) * H + e / H] = s.P[oW2 + e];
+#pragma unroll 8
+    for (int k = 0; k < K; ++k) {
+        const float4 x = lds4(a + k * lda), y = lds4(b + k * ldb);
+        const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                acc[i][j] = fmaf(xs[i], ys[j], acc[i][j]);
+    }
+}
+
+// acc[i][j] += sum over b = 0 .. B-1, in order, of rows a + i sa and c + j sc
+template <int NI, int NJ>
+__device__ __forceinline__ void tile_dots(float (&acc)[NI][NJ], const float *a, int sa, const float *c, int sc, int B)
+{
+    int b = 0;
+#pragma unroll 2
+    for (; b + 4 <= B; b += 4) {
+        float4 x[NI], y[NJ];
+#pragma unroll
+        for (int i = 0; i < NI; ++i)
+            x[i] = lds4(a + i * sa + b);
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+            y[j] = lds4(c + j * sc + b);
+#pragma unroll
+        for (int i = 0; i < NI; ++i)
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                acc[i][j] = fmaf(x[i].x, y[j].x, acc[i][j]);
+                acc[i][j] = fmaf(x[i].y, y[j].y, acc[i][j]);
+                acc[i][j] = fmaf(x[i].z, y[j].z, acc[i][j]);
+                acc[i][j] = fmaf(x[i].w, y[j].w, acc[i][j]);
+            }
+    }
+    for (; b < B; ++b)
+#pragma unroll
+        for (int i = 0; i < NI; ++i)
+#pragma unroll
+            for (int j = 0; j < NJ; ++j)
+                acc[i][j] = fmaf(a[i * sa + b], c[j * sc + b], acc[i][j]);
+}
+
+// sum over b = 0 .. B-1, in order, of a row
+__device__ __forceinline__ float row_sum(const float *a, int B)
+{
+    float acc = 0.f;
+    int b = 0;
+#pragma unroll 4
+    for (; b + 4 <= B; b += 4) {
+        const float4 x = lds4(a + b);
+        acc += x.x;
+        acc += x.y;
+        acc += x.z;
+        acc += x.w;
+    }
+    for (; b < B; ++b)
+        acc += a[b];
+    return acc;
+}
+
+// where the forward and backward products read parameter e
+__device__ __forceinline__ void train_store(TrainShared &s, int e, float p)
+{
+    if (e < ob1) {
+        s.w1t[(e % I) * H + e / I] = p;
+    } else if (e < oW2) {
+        s.b1[e - ob1] = p;
+    } else if (e < ob2) {
+        const int w = e - oW2;
+        s.w2t[(w % H) * H + w / H] = p;
+        s.w2[w] = p;
+    } else if (e < oW3) {
+        s.b2[e - ob2] = p;
+    } else if (e < ob3) {
+        s.w3[e - oW3] = p;
+    } else {
+        s.b3[e - ob3] = p;
+    }
 }
 
 __global__ void __launch_bounds__(kTrainThreads, 1)
@@ -308,130 +404,197 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
 {
     extern __shared__ __align__(16) unsigned char raw[];
     TrainShared &s = *reinterpret_cast<TrainShared *>(raw);
-    const int tid = threadIdx.x, nt = blockDim.x;
-    for (int e = tid; e < NP; e += nt)
-        s.P[e] = Pg[e];
-    __syncthreads();
-    refresh_transposed(s);
+    const int tid = threadIdx.x;
+    // 4 x 4 tiles of the products over features x samples: a warp takes 4 feature quads
+    // x 8 sample quads; tiles wholly past the batch are skipped
+    const int tu = (((tid >> 3) & 3) | (tid >> 7) << 2) * 4, tb = ((tid & 7) | ((tid >> 5) & 3) << 3) * 4;
+    const bool tile = tb < B;
+    float p[kTrainPer], m[kTrainPer], v[kTrainPer], xn[kTrainX], tn = 0.f;
+#pragma unroll
+    for (int r = 0; r < kTrainPer; ++r) {
+        const int e = tid + r * kTrainThreads;
+        p[r] = e < NP ? Pg[e] : 0.f;
+        m[r] = e < NP ? M[e] : 0.f;
+        v[r] = e < NP ? Vv[e] : 0.f;
+        if (e < NP)
+            train_store(s, e, p[r]);
+    }
+    // the next step's rows are in flight during the present one
+    auto fetch = [&](int64_t st) {
+        const int64_t first = (st * B) % N;
+#pragma unroll
+        for (int r = 0; r < kTrainX; ++r) {
+            const int e = tid + r * kTrainThreads;
+            xn[r] = e < B * I ? X[((first + e / I) % N) * I + e % I] : 0.f;
+        }
+        if (tid < B * O)
+            tn = T[((first + tid / O) % N) * O + tid % O];
+    };
     const float invB = 1.f / (float)B;
+    fetch(0);
     for (int64_t st = 0; st < steps; ++st) {
-        for (int e = tid; e < B * I; e += nt)
-            s.x[e] = X[((st * B + e / I) % N) * I + e % I];
-        for (int e = tid; e < B * O; e += nt)
-            s.t[e] = T[((st * B + e / O) % N) * O + e % O];
+#pragma unroll
+        for (int r = 0; r < kTrainX; ++r) {
+            const int e = tid + r * kTrainThreads;
+            s.xt[e % I][e / I] = xn[r];
+        }
+        if (tid < B * O)
+            s.t[tid] = tn;
         if (tid == 0)
             s.loss = 0.f;
+        if (st + 1 < steps)
+            fetch(st + 1);
         __syncthreads();
-        // A1[b][u] = b1[u] + sum_i W1[u][i] x[b][i]
-        for (int e = tid; e < B * H; e += nt) {
-            const int b = e / H, u = e % H;
-            float acc = s.P[ob1 + u];
+        // A1[u][b] = b1[u] + sum_i W1[u][i] x[b][i], then A2 from h1 in the same way
+        if (tile) {
+            float acc[4][4];
 #pragma unroll
-            for (int i = 0; i < I; ++i)
-                acc = fmaf(s.w1t[i * H + u], s.x[b * I + i], acc);
-            s.a1[e] = acc;
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    acc[i][j] = s.b1[tu + i];
+            tile_rows(acc, s.w1t + tu, H, &s.xt[0][tb], kTrainRow, I);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                *reinterpret_cast<float4 *>(&s.h1[tu + i][tb]) = make_float4(
+                    fmaxf(acc[i][0], 0.f), fmaxf(acc[i][1], 0.f), fmaxf(acc[i][2], 0.f), fmaxf(acc[i][3], 0.f));
         }
         __syncthreads();
-        // A2[b][u] = b2[u] + sum_i W2[u][i] relu(A1[b][i])
-        for (int e = tid; e < B * H; e += nt) {
-            const int b = e / H, u = e % H;
-            float acc = s.P[ob2 + u];
-#pragma unroll 8
-            for (int i = 0; i < H; ++i)
-                acc = fmaf(s.w2t[i * H + u], fmaxf(s.a1[b * H + i], 0.f), acc);
-            s.a2[e] = acc;
+        if (tile) {
+            float acc[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    acc[i][j] = s.b2[tu + i];
+            tile_rows(acc, s.w2t + tu, H, &s.h1[0][tb], kTrainRow, H);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                *reinterpret_cast<float4 *>(&s.h2[tu + i][tb]) = make_float4(
+                    fmaxf(acc[i][0], 0.f), fmaxf(acc[i][1], 0.f), fmaxf(acc[i][2], 0.f), fmaxf(acc[i][3], 0.f));
         }
         __syncthreads();
-        // y[b][o], dY = (y - t) / B, loss
-        for (int e = tid; e < B * O; e += nt) {
-            const int b = e / O, o = e % O;
-            float acc = s.P[ob3 + o];
+        // y[b][o] (each lane starts its sum at its own unit), dY = (y - t) / B, loss
+        float loss = 0.f;
+        if (tid < B * O) {
+            const int b = tid / O, o = tid % O;
+            float acc = s.b3[o];
+#pragma unroll 16
             for (int j = 0; j < H; ++j) {
-                const int u = (j + (tid & 31)) & (H - 1);  // skewed so lanes hit distinct banks
-                acc = fmaf(s.P[oW3 + o * H + u], fmaxf(s.a2[b * H + u], 0.f), acc);
+                const int u = (j + (tid & 31)) & (H - 1);
+                acc = fmaf(s.w3[o * H + u], s.h2[u][b], acc);
             }
-            const float err = acc - s.t[e];
-            s.dy[e] = err * invB;
-            atomicAdd(&s.loss, 0.5f * err * err * invB);
+            const float err = acc - s.t[tid];
+            s.dy[o][b] = err * invB;
+            loss = 0.5f * err * err * invB;
+        }
+        if (loss_out && tid < 2 * kTrainMaxB) {
+            loss = warp_sum(loss);  // (a shared-memory float atomic per sample queued 256 deep)
+            if ((tid & 31) == 0)
+                atomicAdd(&s.loss, loss);
         }
         __syncthreads();
-        // gW3[o][u], gb3[o]; dA2[b][u]
-        for (int e = tid; e < O * H; e += nt) {
-            const int o = e / H, u = e % H;
-            float acc = 0.f;
-            for (int b = 0; b < B; ++b)
-                acc = fmaf(s.dy[b * O + o], fmaxf(s.a2[b * H + u], 0.f), acc);
-            s.G[oW3 + e] = acc;
-        }
-        if (tid < O) {
-            float acc = 0.f;
-            for (int b = 0; b < B; ++b)
-                acc += s.dy[b * O + tid];
-            s.G[ob3 + tid] = acc;
-        }
-        for (int e = tid; e < B * H; e += nt) {
-            const int b = e / H, u = e % H;
-            const float g = s.P[oW3 + u] * s.dy[b * O] + s.P[oW3 + H + u] * s.dy[b * O + 1];
-            s.da[e] = s.a2[e] > 0.f ? g : 0.f;
-        }
-        __syncthreads();
-        // gW2[u][i] = sum_b dA2[b][u] relu(A1[b][i]); gb2[u]
-        for (int e = tid; e < H * H; e += nt) {
-            const int u = e / H, i = e % H;
-            float acc = 0.f;
-            for (int b = 0; b < B; ++b)
-                acc = fmaf(s.da[b * H + u], fmaxf(s.a1[b * H + i], 0.f), acc);
-            s.G[oW2 + e] = acc;
-        }
-        for (int u = tid; u < H; u += nt) {
-            float acc = 0.f;
-            for (int b = 0; b < B; ++b)
-                acc += s.da[b * H + u];
-            s.G[ob2 + u] = acc;
+        // dA2[u][b]
+        if (tile) {
+            const float4 d0 = lds4(&s.dy[0][tb]), d1 = lds4(&s.dy[1][tb]);
+            const float dy0[4] = {d0.x, d0.y, d0.z, d0.w}, dy1[4] = {d1.x, d1.y, d1.z, d1.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int u = tu + i;
+                const float4 h = lds4(&s.h2[u][tb]);
+                const float hs[4] = {h.x, h.y, h.z, h.w};
+                float d[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float g = s.w3[u] * dy0[j] + s.w3[H + u] * dy1[j];
+                    d[j] = hs[j] > 0.f ? g : 0.f;
+                }
+                *reinterpret_cast<float4 *>(&s.da2[u][tb]) = make_float4(d[0], d[1], d[2], d[3]);
+            }
         }
         __syncthreads();
-        // dA1[b][i] = relu'(A1[b][i]) sum_u W2[u][i] dA2[b][u]  (into a2)
-        for (int e = tid; e < B * H; e += nt) {
-            const int b = e / H, i = e % H;
-            float acc = 0.f;
-#pragma unroll 8
-            for (int u = 0; u < H; ++u)
-                acc = fmaf(s.P[oW2 + u * H + i], s.da[b * H + u], acc);
-            s.a2[e] = s.a1[e] > 0.f ? acc : 0.f;
+        // the first half of the threads: gW2[u][i] = sum_b dA2[u][b] h1[i][b]; the other
+        // half: dA1[i][b] = relu'(A1) sum_u W2[u][i] dA2[u][b], then gW3, gb2 and gb3
+        if (tid < 256) {
+            // rows u, u + 8, u + 16, u + 24 of dA2 and i, i + 8, ... of h1
+            const int u = ((tid >> 3) & 7) | (tid >> 6 & 1) << 5, i0 = (tid & 7) | (tid >> 7) << 5;
+            float acc[4][4] = {};
+            tile_dots<4, 4>(acc, s.da2[u], 8 * kTrainRow, s.h1[i0], 8 * kTrainRow, B);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    s.G[oW2 + (u + 8 * i) * H + i0 + 8 * j] = acc[i][j];
+        } else {
+            for (int e = tid - 256; e < 512; e += 256) {
+                const int i0 = (((e >> 3) & 3) | (e >> 7) << 2) * 4, b = ((e & 7) | ((e >> 5) & 3) << 3) * 4;
+                if (b >= B)
+                    continue;
+                float acc[4][4] = {};
+                tile_rows(acc, s.w2 + i0, H, &s.da2[0][b], kTrainRow, H);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 h = lds4(&s.h1[i0 + i][b]);
+                    *reinterpret_cast<float4 *>(&s.da1[i0 + i][b]) =
+                        make_float4(h.x > 0.f ? acc[i][0] : 0.f, h.y > 0.f ? acc[i][1] : 0.f,
+                                    h.z > 0.f ? acc[i][2] : 0.f, h.w > 0.f ? acc[i][3] : 0.f);
+                }
+            }
+            const int w = tid - 256;
+            if (w < O * H) {
+                float acc[1][1] = {};
+                tile_dots<1, 1>(acc, s.dy[w / H], 0, s.h2[w % H], 0, B);
+                s.G[oW3 + w] = acc[0][0];
+            } else if (w < O * H + H) {
+                s.G[ob2 + w - O * H] = row_sum(s.da2[w - O * H], B);
+            } else if (w < O * H + H + O) {
+                s.G[ob3 + w - O * H - H] = row_sum(s.dy[w - O * H - H], B);
+            }
         }
         __syncthreads();
-        // gW1[u][i] = sum_b dA1[b][u] x[b][i]; gb1[u]
-        for (int e = tid; e < H * I; e += nt) {
-            const int u = e / I, i = e % I;
-            float acc = 0.f;
-            for (int b = 0; b < B; ++b)
-                acc = fmaf(s.a2[b * H + u], s.x[b * I + i], acc);
-            s.G[oW1 + e] = acc;
-        }
-        for (int u = tid; u < H; u += nt) {
-            float acc = 0.f;
-            for (int b = 0; b < B; ++b)
-                acc += s.a2[b * H + u];
-            s.G[ob1 + u] = acc;
+        // gW1[u][i] = sum_b dA1[u][b] x[i][b]; gb1[u]
+        if (tid < H * I / 4) {
+            const int u = ((tid >> 3) & 7) | (tid >> 6 & 1) << 5 | (tid >> 7) << 3, i = tid & 7;
+            // rows u, u + 16 of dA1 and i, i + 8 of x
+            float acc[2][2] = {};
+            tile_dots<2, 2>(acc, s.da1[u], 16 * kTrainRow, s.xt[i], 8 * kTrainRow, B);
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+                    s.G[oW1 + (u + 16 * a) * I + i + 8 * c] = acc[a][c];
+        } else if (tid < H * I / 4 + H) {
+            s.G[ob1 + tid - H * I / 4] = row_sum(s.da1[tid - H * I / 4], B);
         }
         __syncthreads();
         const int64_t t = t0 + st + 1;
         const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
-        for (int e = tid; e < NP; e += nt) {
-            float p = s.P[e], m = M[e], v = Vv[e];
-            adam1(p, s.G[e], m, v, lr, b1, b2, eps, c1, c2);
-            s.P[e] = p;
-            M[e] = m;
-            Vv[e] = v;
+#pragma unroll
+        for (int r = 0; r < kTrainPer; ++r) {
+            const int e = tid + r * kTrainThreads;
+            if (e < NP) {
+                // the fused forms adam1 compiles to where it was measured, written out: a
+                // rounding more or less would drift over the steps
+                const float g = s.G[e];
+                m[r] = fmaf(b1, m[r], (1.f - b1) * g);
+                v[r] = fmaf(b2, v[r], __fmul_rn((1.f - b2) * g, g));
+                p[r] -= lr * (m[r] / c1) / (sqrtf(v[r] / c2) + eps);
+                train_store(s, e, p[r]);
+            }
         }
         if (tid == 0 && loss_out)
             loss_out[st] = s.loss;
         __syncthreads();
-        refresh_transposed(s);
     }
-    __syncthreads();
-    for (int e = tid; e < NP; e += nt)
-        Pg[e] = s.P[e];
+#pragma unroll
+    for (int r = 0; r < kTrainPer; ++r) {
+        const int e = tid + r * kTrainThreads;
+        if (e < NP) {
+            Pg[e] = p[r];
+            M[e] = m[r];
+            Vv[e] = v[r];
+        }
+    }
 }
 
 // bfloat16 evaluation: weights and inputs rounded to bfloat16, float32

@@ -621,7 +621,7 @@ __global__ void knn_emit_kernel(int64_t nq, const unsigned long long *__restrict
 // TMA ring) that both row blocks share.  Shared memory holds the operands
 // K-major in 128-byte-swizzled atoms (8 rows x 64 bfloat16).  Warp 9 allocates
 // the 512 TMEM columns: for each row block two 128 x 128 float32 accumulators
-// (tiles alternate between them).  Its lane 0 issues tcgen05.mma (M = 128,
+// (tiles alternate between them).  One lane of it issues tcgen05.mma (M = 128,
 // N = 128, K = 16 per instruction, both row blocks per K step) and commits to
 // mbarriers that free the smem stage and hand the accumulators to the epilogue.
 // Warp 8 lane 0 issues the TMA loads.
@@ -736,16 +736,29 @@ __host__ __device__ constexpr uint32_t umma_idesc(int M, int N)
 {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ void umma_bf16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc)
+// One lane of a converged warp.
+__device__ __forceinline__ uint32_t elect_one()
 {
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(dtmem),
-                 "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
+    uint32_t x;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xFFFFFFFF;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(x));
+    return x;
+}
+// The MMA and the commit are issued where `lead` is set, by a warp that runs converged
+// with the same operands in every lane: operands of a single diverged lane went through
+// a register transfer each (24 per MMA; 87 cycles between MMAs that take 64).
+__device__ __forceinline__ void umma_bf16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc,
+                                          uint32_t lead)
+{
+    asm volatile("{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+                 " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(dtmem),
+                 "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc), "r"(lead)
                  : "memory");
 }
-__device__ __forceinline__ void umma_commit(uint64_t *bar)
+__device__ __forceinline__ void umma_commit(uint64_t *bar, uint32_t lead)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
+    asm volatile("{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+                 " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(smem_u32(bar)),
+                 "r"(lead)
                  : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -888,7 +901,9 @@ __device__ void tc_epilogue(uint64_t *accf, uint64_t *acce, uint32_t tmem, int w
         // term an exact integer or half-integer for byte-valued inputs (approximate in
         // the split float form, whose survivors are rescored)
         const float tr = 0.5f * (qnr - thr);
-        const int cb0 = (int)col0, left = (int)(n - col0);  // columns of the tile below n: 128 or, in the last, fewer
+        // columns of the tile below n (fewer than 128 in the last; none for rows that are no
+        // query, whose accumulators may never have been written)
+        const int cb0 = (int)col0, left = row_ok ? (int)min(n - col0, (int64_t)TC_N) : 0;
         const int64_t sd = self - col0;
         const int sj0 = sd >= 0 && sd < TC_N ? (int)sd : -1;
         const float4 *h4 = reinterpret_cast<const float4 *>(xh + (EPI == EPI_NORMS ? col0 : 0));
@@ -1033,43 +1048,48 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
     } else if (warp == 9) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc(TC_M, TC_N);
-            int64_t done = 0;
-            bool ok = mbar_wait(abar, 0, err, 2);
-            for (int64_t t = 0; ok && t < tiles; ++t) {
-                const int s = (int)(t % L::STAGES), b = (int)(t & 1);
-                if (!mbar_wait(&full[s], (uint32_t)((t / L::STAGES) & 1), err, 3))
-                    break;
-                if (t >= 2 && !mbar_wait(&acce[b], (uint32_t)(((t >> 1) & 1) ^ 1), err, 4))
-                    break;
-                tc_fence_after();
-                const uint32_t bb = smem_u32(sB + s * L::B_STAGE);
+        constexpr uint32_t idesc = umma_idesc(TC_M, TC_N);
+        const uint32_t lead = elect_one();
+        const uint64_t a0 = umma_desc(smem_u32(sA)), b0 = umma_desc(smem_u32(sB));
+        int64_t done = 0;
+        bool ok = __all_sync(0xffffffffu, mbar_wait(abar, 0, err, 2));
+        int s = 0;
+        uint32_t sp = 0;  // ring stage and its parity
+        for (int64_t t = 0; ok && t < tiles; ++t) {
+            const int b = (int)(t & 1);
+            if (!__all_sync(0xffffffffu, mbar_wait(&full[s], sp, err, 3)))
+                break;
+            if (t >= 2 && !__all_sync(0xffffffffu, mbar_wait(&acce[b], (uint32_t)(((t >> 1) & 1) ^ 1), err, 4)))
+                break;
+            tc_fence_after();
+            const uint64_t bt = b0 + (uint32_t)(s * (L::B_STAGE >> 4));
 #pragma unroll
-                for (int rb = 0; rb < TC_RB; ++rb) {
-                    if (rb >= nrb)
-                        break;
-                    const uint32_t aa = smem_u32(sA + rb * (KA - 1) * L::A_ATOM);
-                    const uint32_t dt = tmem + (uint32_t)((rb * 2 + b) * TC_N);
+            for (int rb = 0; rb < TC_RB; ++rb) {
+                if (rb >= nrb)
+                    break;
+                const uint64_t at = a0 + (uint32_t)(rb * (KA - 1) * (L::A_ATOM >> 4));
+                const uint32_t dt = tmem + (uint32_t)((rb * 2 + b) * TC_N);
 #pragma unroll
-                    for (int kk = 0; kk < 4 * (KA - 1); ++kk) {
-                        const uint32_t off = (uint32_t)((kk & 3) * 32);  // 16 bf16 = 32 bytes inside the atom
-                        const uint64_t ad = umma_desc(aa + (kk >> 2) * L::A_ATOM + off);
-                        const uint64_t bd = umma_desc(bb + (kk >> 2) * L::B_ATOM + off);
-                        umma_bf16(dt, ad, bd, idesc, kk > 0 ? 1u : 0u);
-                    }
-                    // the spare atom's first K step adds -floor(|x|^2 / 2)
-                    umma_bf16(dt, umma_desc(smem_u32(sA + TC_RB * (KA - 1) * L::A_ATOM)),
-                              umma_desc(bb + (KA - 1) * L::B_ATOM), idesc, 1u);
+                for (int kk = 0; kk < 4 * (KA - 1); ++kk) {
+                    const uint32_t off = (uint32_t)((kk & 3) * 32);  // 16 bf16 = 32 bytes inside the atom
+                    umma_bf16(dt, at + (((kk >> 2) * L::A_ATOM + off) >> 4), bt + (((kk >> 2) * L::B_ATOM + off) >> 4),
+                              idesc, kk > 0 ? 1u : 0u, lead);
                 }
-                umma_commit(&empty[s]);
-                umma_commit(&accf[b]);
-                done = t + 1;
+                // the spare atom's first K step adds -floor(|x|^2 / 2)
+                umma_bf16(dt, a0 + (uint32_t)(TC_RB * (KA - 1) * (L::A_ATOM >> 4)),
+                          bt + (uint32_t)((KA - 1) * (L::B_ATOM >> 4)), idesc, 1u, lead);
             }
-            // the MMAs issued so far complete before TMEM is freed (bounded)
-            if (done > 0)
-                mbar_drain(&accf[(done - 1) & 1], (uint32_t)(((done - 1) >> 1) & 1), err, 7);
+            umma_commit(&empty[s], lead);
+            umma_commit(&accf[b], lead);
+            done = t + 1;
+            if (++s == L::STAGES) {
+                s = 0;
+                sp ^= 1;
+            }
         }
+        // the MMAs issued so far complete before TMEM is freed (bounded)
+        if (done > 0)
+            mbar_drain(&accf[(done - 1) & 1], (uint32_t)(((done - 1) >> 1) & 1), err, 7);
     } else {
         // ------------------------------------------------ epilogue (warps 0-7)
         tc_epilogue<KC, EPI_BYTE>(accf, acce, tmem, warp, lane, row0, nq, n, tm, k - 1, self_offset, nullptr, par, qn,
@@ -1190,45 +1210,51 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
     } else if (warp == 9) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t idesc = umma_idesc(TC_M, TC_N);
-            int64_t last = -1;  // the last step whose MMAs were issued (and committed to empty)
-            for (int64_t step = 0; step < steps; ++step) {
-                const int s = (int)(step % TCS_STAGES);
-                const int64_t t = step / nk;
-                const int kc = (int)(step % nk), b = (int)(t & 1);
-                if (!mbar_wait(&full[s], (uint32_t)((step / TCS_STAGES) & 1), err, 3))
-                    break;
-                if (kc == 0 && t >= 2 && !mbar_wait(&acce[b], (uint32_t)(((t >> 1) & 1) ^ 1), err, 4))
-                    break;
-                tc_fence_after();
-                const uint32_t st = smem_u32(base + s * L::STAGE);
+        constexpr uint32_t idesc = umma_idesc(TC_M, TC_N);
+        constexpr uint32_t atom = L::ATOM >> 4;
+        const uint32_t lead = elect_one();
+        const uint64_t r0 = umma_desc(smem_u32(base));
+        int64_t last = -1;  // the last step whose MMAs were issued (and committed to empty)
+        int kc = 0;
+        int64_t t = 0;
+        for (int64_t step = 0; step < steps; ++step) {
+            const int s = (int)(step % TCS_STAGES);
+            const int b = (int)(t & 1);
+            if (!__all_sync(0xffffffffu, mbar_wait(&full[s], (uint32_t)((step / TCS_STAGES) & 1), err, 3)))
+                break;
+            if (kc == 0 && t >= 2 &&
+                !__all_sync(0xffffffffu, mbar_wait(&acce[b], (uint32_t)(((t >> 1) & 1) ^ 1), err, 4)))
+                break;
+            tc_fence_after();
+            const uint64_t st = r0 + (uint32_t)(s * (L::STAGE >> 4));
+            const uint32_t first = kc > 0 ? 1u : 0u;
 #pragma unroll
-                for (int rb = 0; rb < TC_RB; ++rb) {
-                    if (rb >= nrb)
-                        break;
-                    const uint32_t dt = tmem + (uint32_t)((rb * 2 + b) * TC_N);
+            for (int rb = 0; rb < TC_RB; ++rb) {
+                if (rb >= nrb)
+                    break;
+                const uint32_t dt = tmem + (uint32_t)((rb * 2 + b) * TC_N);
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk) {
-                        const uint32_t off = (uint32_t)(kk * 32);  // 16 bf16 = 32 bytes inside the atom
-                        const uint64_t ah = umma_desc(st + rb * L::ATOM + off);
-                        const uint64_t al = umma_desc(st + (2 + rb) * L::ATOM + off);
-                        const uint64_t bh = umma_desc(st + 4 * L::ATOM + off);
-                        const uint64_t bl = umma_desc(st + 5 * L::ATOM + off);
-                        umma_bf16(dt, ah, bh, idesc, (kc > 0 || kk > 0) ? 1u : 0u);
-                        umma_bf16(dt, ah, bl, idesc, 1u);
-                        umma_bf16(dt, al, bh, idesc, 1u);
-                    }
+                for (int kk = 0; kk < 4; ++kk) {
+                    const uint32_t off = (uint32_t)(kk * 2);  // 16 bf16 = 32 bytes inside the atom
+                    const uint64_t ah = st + rb * atom + off, al = st + (2 + rb) * atom + off;
+                    const uint64_t bh = st + 4 * atom + off, bl = st + 5 * atom + off;
+                    umma_bf16(dt, ah, bh, idesc, kk > 0 ? 1u : first, lead);
+                    umma_bf16(dt, ah, bl, idesc, 1u, lead);
+                    umma_bf16(dt, al, bh, idesc, 1u, lead);
                 }
-                umma_commit(&empty[s]);
-                if (kc == nk - 1)
-                    umma_commit(&accf[b]);
-                last = step;
             }
-            // the MMAs issued so far complete before TMEM is freed (bounded)
-            if (last >= 0)
-                mbar_drain(&empty[last % TCS_STAGES], (uint32_t)((last / TCS_STAGES) & 1), err, 7);
+            umma_commit(&empty[s], lead);
+            if (kc == nk - 1)
+                umma_commit(&accf[b], lead);
+            last = step;
+            if (++kc == nk) {
+                kc = 0;
+                ++t;
+            }
         }
+        // the MMAs issued so far complete before TMEM is freed (bounded)
+        if (last >= 0)
+            mbar_drain(&empty[last % TCS_STAGES], (uint32_t)((last / TCS_STAGES) & 1), err, 7);
     } else {
         // ------------------------------------------------ epilogue (warps 0-7)
         tc_epilogue<KC, FOLD ? EPI_FOLD : EPI_NORMS>(accf, acce, tmem, warp, lane, row0, nq, n, tm, KC - 1, self_offset, xh,

@@ -1332,48 +1332,74 @@ __global__ void split_rows_kernel(const float *__restrict__ M, int64_t rows, int
     }
 }
 
-// Sets bit 0 of *flag if any value is not an integer in [0, 255] (byte-valued
-// descriptors: exact in bfloat16, and at d <= 128 every squared norm, dot product,
-// |x|^2 / 2 and distance of the tensor-core path is an exact float32 below 2^23),
-// and bit 1 if any value is not an integer at all.
-__global__ void value_kind_kernel(const float *__restrict__ x, int64_t count, int *flag)
-{
-    unsigned bad = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        const float v = x[i];
-        const bool integer = v == rintf(v);
-        bad |= (integer && v >= 0.f && v <= 255.f) ? 0u : 1u;
-        bad |= integer ? 0u : 2u;
-    }
-    bad = __reduce_or_sync(0xffffffffu, bad);
-    if ((threadIdx.x & 31) == 0 && bad)
-        atomicOr(flag, (int)bad);
-}
-
-// The byte-valued form's operands: row r of M in bfloat16 in columns [0, d) of a
-// row of dpa = dp + 64 (dp = d rounded up to whole K atoms, and a spare one), then in
-// columns dp, dp + 1, dp + 2 either 1.0 (queries: s == nullptr) or the three pieces
-// of -floor(s_r / 2) (base rows; s_r = |x_r|^2, an integer below 2^23): its 8-bit
-// fields times 2^16, 2^8 and 1, each exact in bfloat16; zeros elsewhere.  The MMA
-// then accumulates q.x - floor(|x|^2 / 2) exactly.  Padding d to whole K atoms takes
-// byte rows of any d = 32 .. 128 here from the float32 sweep (30,011 x 100, the whole
-// build: 20.5 -> 9.3 ms); below 32 the ties of small integers would flood the lists.
-__global__ void aug_rows_kernel(const float *__restrict__ M, int64_t rows, int d, int dpa,
-                                const float *__restrict__ s, __nv_bfloat16 *__restrict__ out)
+// One pass over the rows of M for what every sweep needs to know of them (one read of
+// the base instead of three; the whole call at 30,011 x 100: 2.89 -> 2.62 ms):
+// - the squared norms s_r, in norms_kernel's order of sums;
+// - bit 0 of *flag if any value is not an integer in [0, 255] (byte-valued
+//   descriptors: exact in bfloat16, and at d <= 128 every squared norm, dot product,
+//   |x|^2 / 2 and distance of the tensor-core path is an exact float32 below 2^23), and
+//   bit 1 if any value is not an integer at all;
+// - with `out`, as long as no other value has been seen, the byte-valued form's
+//   operands: row r in bfloat16 in columns [0, d) of a row of dpa = dp + 64 (dp = d
+//   rounded up to whole K atoms, and a spare one), then in columns dp, dp + 1, dp + 2
+//   either 1.0 (queries) or the three pieces of -floor(s_r / 2) (base rows; s_r is an
+//   integer below 2^23): its 8-bit fields times 2^16, 2^8 and 1, each exact in
+//   bfloat16; zeros elsewhere.  The MMA then accumulates q.x - floor(|x|^2 / 2) exactly.
+//   Padding d to whole K atoms takes byte rows of any d = 32 .. 128 here from the float32
+//   sweep (30,011 x 100, the whole build: 20.5 -> 9.3 ms); below 32 the ties of small
+//   integers would flood the lists.
+__global__ void prepare_rows_kernel(const float *__restrict__ M, int64_t rows, int d, int dpa, bool base,
+                                    float *__restrict__ norm, __nv_bfloat16 *__restrict__ out, int *flag)
 {
     const int lane = threadIdx.x & 31;
+    auto kind = [](float v) {
+        const bool integer = v == rintf(v);
+        return (integer && v >= 0.f && v <= 255.f ? 0u : 1u) | (integer ? 0u : 2u);
+    };
     for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < rows;
          r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const unsigned h = s ? ((unsigned)s[r]) >> 1 : 0u;
-        for (int j = lane; j < dpa; j += 32) {
-            float v = 0.f;
-            if (j < d)
-                v = M[r * d + j];
-            else if (j >= dpa - 64 && j < dpa - 61) {
-                const int p = j - (dpa - 64);
-                v = !s ? 1.f : -(float)(p == 0 ? (h >> 16) << 16 : p == 1 ? ((h >> 8) & 255u) << 8 : h & 255u);
+        const float4 *p = reinterpret_cast<const float4 *>(M + r * d);
+        float s = 0.f;
+        unsigned bad = 0;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = lane; c < (d >> 2); c += 32) {
+            v = __ldg(p + c);
+            s = fmaf(v.x, v.x, s);
+            s = fmaf(v.y, v.y, s);
+            s = fmaf(v.z, v.z, s);
+            s = fmaf(v.w, v.w, s);
+            bad |= kind(v.x) | kind(v.y) | kind(v.z) | kind(v.w);
+        }
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1)
+            s += __shfl_xor_sync(0xffffffffu, s, off);
+        bad = __reduce_or_sync(0xffffffffu, bad);
+        const int seen = *reinterpret_cast<volatile int *>(flag);
+        if (lane == 0) {
+            norm[r] = s;
+            if (bad & ~(unsigned)seen)
+                atomicOr(flag, (int)bad);
+        }
+        if (!out || ((bad | (unsigned)seen) & 1u))
+            continue;
+        // d <= 128: v is this lane's quad of the row
+        auto bits = [](float x, float y) {
+            const __nv_bfloat162 b = __floats2bfloat162_rn(x, y);
+            return *reinterpret_cast<const unsigned *>(&b);
+        };
+        uint2 *row = reinterpret_cast<uint2 *>(out + r * dpa);
+        const int quads = (dpa - 64) >> 2;
+        if (lane < quads)
+            row[lane] = make_uint2(bits(v.x, v.y), bits(v.z, v.w));
+        if (lane < 16) {
+            float a = 0.f, b = 0.f, c = 0.f;
+            if (lane == 0) {
+                const unsigned h = (unsigned)s >> 1;
+                a = base ? -(float)((h >> 16) << 16) : 1.f;
+                b = base ? -(float)(((h >> 8) & 255u) << 8) : 1.f;
+                c = base ? -(float)(h & 255u) : 1.f;
             }
-            out[r * dpa + j] = __float2bfloat16_rn(v);
+            row[quads + lane] = make_uint2(bits(a, b), bits(c, 0.f));
         }
     }
 }
@@ -1512,10 +1538,8 @@ int launch_tc(const float *X, int64_t n, int d, const float *Q, int64_t nq, int 
     const int gb = num_sms() * 8;
     const int dpa = (d + 63) / 64 * 64 + 64;  // whole K atoms; the extra one carries -floor(|x|^2 / 2)
     const Shares sh = plan_tc(n, d, nq, kc);
-    aug_rows_kernel<<<gb, 256, 0, s>>>(X, n, d, dpa, xn, xb);
-    aug_rows_kernel<<<gb, 256, 0, s>>>(Q, nq, d, dpa, nullptr, qb);
     parity_kernel<<<gb, 256, 0, s>>>(xn, n, (n + TC_N - 1) / TC_N * (TC_N / 32), par);
-    int st = check_launch("onng_knn: bf16 operands");
+    int st = check_launch("onng_knn: parity");
     if (st)
         return st;
     CUtensorMap ma, mb;
@@ -1664,30 +1688,37 @@ extern "C" int onng_knn(const float *X, int64_t n, int32_t d, const float *Q, in
     float *mu = c.take<float>((size_t)d);
     unsigned *par = c.take<unsigned>((size_t)(std::max<int64_t>(n, 1) + TC_N - 1) / TC_N * (TC_N / 32));
     cudaStream_t s = to_cuda(stream);
-    if (n > 0)
-        norms_kernel<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(X, n, d, xn);
-    norms_kernel<<<(unsigned)((nq * 32 + 255) / 256), 256, 0, s>>>(Q, nq, d, qn);
-    int st = check_launch("onng_knn: norms");
-    if (st)
-        return st;
-    // tensor-core paths (at least one full tile of base rows and one row block of
-    // queries, k + 16 <= 128): byte-valued inputs at d = 32 .. 128 exactly; other
-    // non-integer inputs at d >= 32 by the split bfloat16 form.  Integer-valued
-    // inputs otherwise take the SIMT sweep, which ranks them exactly.
-    if (n >= TC_N && nq >= TC_M && kc <= 128 && n <= INT32_MAX - TC_N) {
+    // tensor-core paths (k + 16 <= 128, from one row block of queries): byte-valued inputs
+    // at d = 32 .. 128 exactly; other non-integer inputs at d >= 32 by the split bfloat16
+    // form.  Integer-valued inputs otherwise take the SIMT sweep, which ranks them exactly.
+    const bool tc = nq >= TC_M && n >= TC_N && kc <= 128 && n <= INT32_MAX - TC_N;
+    int st;
+    if (tc) {
         ONNG_CUDA_TRY(cudaMemsetAsync(flags, 0, 64 * sizeof(int), s), "onng_knn: clear flags");
         const int gb = num_sms() * 8;
-        value_kind_kernel<<<gb, 256, 0, s>>>(X, n * d, flags);
-        value_kind_kernel<<<gb, 256, 0, s>>>(Q, nq * d, flags);
+        const bool byte_d = d >= 32 && d <= 128;
+        const int dpa = (d + 63) / 64 * 64 + 64;
+        prepare_rows_kernel<<<gb, 256, 0, s>>>(Q, nq, d, dpa, false, qn, byte_d ? qb : nullptr, flags);
+        prepare_rows_kernel<<<gb, 256, 0, s>>>(X, n, d, dpa, true, xn, byte_d ? xb : nullptr, flags);
+        st = check_launch("onng_knn: rows");
+        if (st)
+            return st;
         int kind = 3;
         ONNG_CUDA_TRY(cudaMemcpyAsync(&kind, flags, sizeof(int), cudaMemcpyDeviceToHost, s), "onng_knn: flag");
         ONNG_CUDA_TRY(cudaStreamSynchronize(s), "onng_knn: value check");
-        if (!(kind & 1) && d >= 32 && d <= 128)
+        if (!(kind & 1) && byte_d)
             return launch_tc(X, n, d, Q, nq, k, kc, self_offset, nbr, len, xn, par, qn, best, bufp, flags + 1, xb,
                              qb, s);
         if ((kind & 2) && d >= 32)
             return launch_tcs(X, n, d, Q, nq, k, kc, self_offset, nbr, len, xh, qn, best, bufp, flags + 1, xb, qb,
                               sums, mu, s);
+    } else {
+        if (n > 0)
+            norms_kernel<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(X, n, d, xn);
+        norms_kernel<<<(unsigned)((nq * 32 + 255) / 256), 256, 0, s>>>(Q, nq, d, qn);
+        st = check_launch("onng_knn: norms");
+        if (st)
+            return st;
     }
     switch (kc) {
     case 32: return launch<32>(X, n, d, Q, nq, k, self_offset, nbr, len, xn, qn, best, bufp, s);

@@ -65,9 +65,8 @@ __global__ void norms_kernel(const float *__restrict__ X, int64_t n, int d, floa
         out[row] = s;
 }
 
-// Compact warp sorts for the sweeps' epilogues: the stage loops run at run
-// time (only the loop over a lane's registers is unrolled), so the code stays
-// small enough for the instruction cache next to the epilogue's hot loop.
+// Compact warp merge of lists (knn_merge_kernel): the stage loop runs at run time, only
+// the loop over a lane's registers is unrolled.
 // Element e = i * 32 + lane lives in v[i] of lane `lane`.
 
 // compare-exchange of registers i and i ^ JR (partners 32 JR elements apart),
@@ -115,17 +114,6 @@ __device__ __forceinline__ void bitonic_step(unsigned long long (&v)[N], int lan
     }
 }
 
-// ascending sort of 32 N keys
-template <int N> __device__ void warp_sort_compact(unsigned long long (&v)[N], int lane)
-{
-    static_assert(N == 1 || N == 2 || N == 4 || N == 8, "N in {1, 2, 4, 8}");
-#pragma unroll 1
-    for (int size = 2; size <= 32 * N; size <<= 1)
-#pragma unroll 1
-        for (int j = size >> 1; j > 0; j >>= 1)
-            bitonic_step<N>(v, lane, size, j);
-}
-
 // ascending merge of a bitonic sequence of 32 N keys (one bitonic merge pass with
 // every element's direction ascending)
 template <int N> __device__ void warp_merge_compact(unsigned long long (&v)[N], int lane)
@@ -135,55 +123,96 @@ template <int N> __device__ void warp_merge_compact(unsigned long long (&v)[N], 
         bitonic_step<N>(v, lane, 64 * N, j);
 }
 
+// One exchange of a bitonic network between lanes: the lower of the two lanes JL apart
+// keeps the smaller key where `up`.
+template <int JL> __device__ __forceinline__ void lane_cas(unsigned long long &v, bool up, int lane)
+{
+    const unsigned long long o = __shfl_xor_sync(0xffffffffu, v, JL);
+    const bool keep_min = ((lane & JL) == 0) == up;
+    v = (o < v) == keep_min ? o : v;
+}
+__device__ __forceinline__ void reg_cas(unsigned long long &a, unsigned long long &b, bool up)
+{
+    const unsigned long long x = a, y = b;
+    const bool swap = (y < x) == up;
+    a = swap ? y : x;
+    b = swap ? x : y;
+}
+// steps of distance 2 JL .. 2 and 1 elements on pairs (element 2 lane + register)
+template <int JL> __device__ __forceinline__ void pair_steps(unsigned long long (&v)[2], bool up, int lane)
+{
+    if constexpr (JL > 0) {
+        lane_cas<JL>(v[0], up, lane);
+        lane_cas<JL>(v[1], up, lane);
+        pair_steps<JL / 2>(v, up, lane);
+    } else {
+        reg_cas(v[0], v[1], up);
+    }
+}
+
 // The warp merges row gr's cnt buffered keys into its sorted best list of KC
 // keys and returns the new threshold: the distance of list entry kth (< KC).
+//
+// A merge holds up its whole CTA (the next tile's accumulators stay taken), so its
+// latency counts: element 64 h + 2 lane + r of the list sits in register m[h][r] of
+// `lane`, which makes every distance of 1 and of 64 or more an exchange of registers,
+// and the buffer goes in 64 keys at a time, sorted descending: the smaller of each pair
+// (list's last 64, sorted keys) and the rest of the list are a bitonic sequence holding
+// the KC smallest.  The network is unrolled: 15 of its 21 sort and 5 of its 7 merge
+// steps cross lanes.  1M x 128 bytes, k = 100 (about 20 merges a row): 344 -> 277 ms
+// against loops over the steps with element 32 r + lane (9,800 cycles a merge, now 5,900
+// with eight warps at it).
 template <int KC>
 __device__ __noinline__ float merge_row(int64_t gr, int cnt, int kth, unsigned long long *__restrict__ best,
                                            const unsigned long long *__restrict__ buf, int lane)
 {
-    static_assert(KC <= BUF && BUF == 256, "the buffer sort holds 256 keys");
-    constexpr int PB = KC / 32;
-    unsigned long long a[8];
+    static_assert(BUF % 64 == 0 && (KC & (KC - 1)) == 0, "whole chunks and a power-of-two list");
+    constexpr int H = KC < 64 ? 1 : KC / 64;
+    ulonglong2 *const list = reinterpret_cast<ulonglong2 *>(best + gr * KC) + lane;
+    const ulonglong2 *const row = reinterpret_cast<const ulonglong2 *>(buf + gr * BUF) + lane;
+    const bool held = KC >= 64 || lane < KC / 2;  // a list of 32 is the first half of one of 64
+    unsigned long long m[H][2];
+    __syncwarp();  // the row's own thread wrote the buffer
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int e = i * 32 + lane;
-        a[i] = e < cnt ? buf[gr * BUF + e] : EMPTY_KEY;
+    for (int h = 0; h < H; ++h) {
+        const ulonglong2 b = held ? list[h * 32] : make_ulonglong2(EMPTY_KEY, EMPTY_KEY);
+        m[h][0] = b.x;
+        m[h][1] = b.y;
     }
-    // sort the smallest power-of-two prefix holding the cnt keys (the rest is +inf)
-    if (cnt <= 64) {
-        unsigned long long t[2] = {a[0], a[1]};
-        warp_sort_compact<2>(t, lane);
-        a[0] = t[0];
-        a[1] = t[1];
-    } else if (cnt <= 128) {
-        unsigned long long t[4] = {a[0], a[1], a[2], a[3]};
-        warp_sort_compact<4>(t, lane);
+#pragma unroll 1
+    for (int o = 0; o < cnt; o += 64) {
+        const ulonglong2 b = row[o >> 1];
+        unsigned long long a[2] = {o + 2 * lane < cnt ? b.x : EMPTY_KEY, o + 2 * lane + 1 < cnt ? b.y : EMPTY_KEY};
+        reg_cas(a[0], a[1], (lane & 1) == 0);
+        pair_steps<1>(a, (lane & 2) == 0, lane);
+        pair_steps<2>(a, (lane & 4) == 0, lane);
+        pair_steps<4>(a, (lane & 8) == 0, lane);
+        pair_steps<8>(a, (lane & 16) == 0, lane);
+        pair_steps<16>(a, false, lane);
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            a[i] = t[i];
-    } else {
-        warp_sort_compact<8>(a, lane);
+        for (int r = 0; r < 2; ++r)
+            m[H - 1][r] = a[r] < m[H - 1][r] ? a[r] : m[H - 1][r];
+#pragma unroll
+        for (int jh = H / 2; jh > 0; jh /= 2)
+#pragma unroll
+            for (int h = 0; h < H; ++h)
+                if (!(h & jh)) {
+                    reg_cas(m[h][0], m[h | jh][0], true);
+                    reg_cas(m[h][1], m[h | jh][1], true);
+                }
+#pragma unroll
+        for (int h = 0; h < H; ++h)
+            pair_steps<16>(m[h], true, lane);
     }
-    unsigned long long bv[PB], m[PB];
+    unsigned long long kv = m[0][0];
 #pragma unroll
-    for (int i = 0; i < PB; ++i)
-        bv[i] = best[gr * KC + i * 32 + lane];
-    // half-cleaner of (a[0 .. KC), reversed best): the smaller of each pair is a
-    // bitonic sequence holding the KC smallest keys
-#pragma unroll
-    for (int i = 0; i < PB; ++i) {
-        const unsigned long long br = __shfl_sync(0xffffffffu, bv[PB - 1 - i], 31 - lane);
-        m[i] = a[i] < br ? a[i] : br;
+    for (int h = 0; h < H; ++h) {
+        if (held)
+            list[h * 32] = make_ulonglong2(m[h][0], m[h][1]);
+        if (kth >> 6 == h)
+            kv = kth & 1 ? m[h][1] : m[h][0];
     }
-    warp_merge_compact<PB>(m, lane);
-#pragma unroll
-    for (int i = 0; i < PB; ++i)
-        best[gr * KC + i * 32 + lane] = m[i];
-    unsigned long long kv = m[0];
-#pragma unroll
-    for (int i = 1; i < PB; ++i)
-        kv = (kth >> 5) == i ? m[i] : kv;
-    return key_dist(__shfl_sync(0xffffffffu, kv, kth & 31));
+    return key_dist(__shfl_sync(0xffffffffu, kv, (kth >> 1) & 31));
 }
 
 // Which share of a sweep a CTA takes.  The row blocks below `main` are swept by gm
@@ -640,7 +669,9 @@ __global__ void knn_emit_kernel(int64_t nq, const unsigned long long *__restrict
 // where TMEM is freed.
 constexpr int TC_M = 128, TC_N = 128, TC_BUF = BUF;
 constexpr int TC_RB = 2;                    // 128-row blocks per CTA
-constexpr int TC_EAGER = 64;                // buffered keys that trigger a merge
+// Buffered keys that trigger a merge: with the last tile's hits they mostly still fit one
+// chunk of 64 (64: 281, 56: 277, 48: 281, 32: 295 ms at 1M x 128 bytes, k = 100).
+constexpr int TC_EAGER = 56;
 constexpr int TC_ROWS = TC_M * TC_RB;       // query rows per CTA
 constexpr int TC_EPI = 256;                 // epilogue threads (8 warps), one per row
 constexpr int TC_THREADS = TC_EPI + 64;     // + TMA warp + MMA warp

@@ -850,10 +850,12 @@ enum { EPI_BYTE, EPI_FOLD, EPI_NORMS };
 // One 32-column chunk of a row: f[j] is column cb + j.  The maxima of eight groups of
 // four columns decide which groups any row of the warp needs; their hits are appended
 // from registers (static indices: a group is four predicated appends).  At 1M x 128
-// bytes, k = 100, two thirds of the chunks hold a hit of some row, and reading hit
-// columns back from TMEM one by one set the pace: 369 -> 352 ms.  A vote per group
-// instead of the one reduction, unrolled over the tile's four chunks, took 627 ms (code
-// size and branches).
+// bytes, k = 100, two thirds of the chunks hold a hit of some row, and the branches over
+// the groups set the pace (about 20 cycles each): tested by halves first, most chunks
+// branch six times instead of eight, 277 -> 263 ms.  Reading hit columns back from TMEM
+// one by one is slower by a twentieth; four groups of eight columns take 267 ms, sixteen
+// of two 317, a jump by group number or anything else that writes f twice as long (the
+// next chunk's TMEM load then no longer runs ahead).
 // sj = the row's own column in the chunk (self-joins), nl = columns of the chunk below n,
 // odd = the parity bits (EPI_BYTE).
 template <int EPI>
@@ -873,14 +875,19 @@ __device__ __forceinline__ void tc_chunk(const float (&f)[32], float tr, float q
         groups |= ((EPI == EPI_BYTE ? m[i] >= tr : m[i] > tr) ? 1u : 0u) << i;
     groups = __reduce_or_sync(0xffffffffu, groups);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        if (!(groups >> i & 1u))
+    for (int h = 0; h < 8; h += 4) {
+        if (!(groups >> h & 15u))
             continue;
 #pragma unroll
-        for (int j = i; j < 32; j += 8) {
-            const float a = EPI == EPI_BYTE && (odd >> j & 1u) ? f[j] - 0.5f : f[j];
-            if ((EPI == EPI_BYTE ? a >= tr : a > tr) && j != sj && j < nl)
-                brow[cnt++] = pack_key(fmaxf(qnr - 2.f * a, 0.f), cb + j);
+        for (int i = h; i < h + 4; ++i) {
+            if (!(groups >> i & 1u))
+                continue;
+#pragma unroll
+            for (int j = i; j < 32; j += 8) {
+                const float a = EPI == EPI_BYTE && (odd >> j & 1u) ? f[j] - 0.5f : f[j];
+                if ((EPI == EPI_BYTE ? a >= tr : a > tr) && j != sj && j < nl)
+                    brow[cnt++] = pack_key(fmaxf(qnr - 2.f * a, 0.f), cb + j);
+            }
         }
     }
 }

@@ -1,12 +1,12 @@
 // Exact k-nearest-neighbour lists (the exact kNN graph that replaces the
 // paper's approximate graph, Sec. 2.6) without materialising the n x n matrix.
 //
-// knn_tile_kernel: a CTA owns 128 query rows and sweeps all base columns in
-// tiles of 128.  The tile of squared distances |q|^2 + |x|^2 - 2 q.x is formed
-// in registers (8 x 8 per thread, float32 FMA).  Entries below the row's
+// knn_tile_kernel: a CTA owns 16, 32, 64 or 128 query rows and sweeps its share of the
+// base columns in tiles of 128.  The tile of squared distances |q|^2 + |x|^2 - 2 q.x is
+// formed in registers (up to 8 x 8 per thread, packed float32 FMA).  Entries below the row's
 // running threshold are appended to a per-row candidate buffer in global
 // memory (mostly L2); when a buffer may not absorb another tile it is merged
-// with the row's best list (a warp-wide bitonic sort in registers) and the
+// with the row's best list (merge_row) and the
 // threshold drops to the list's last entry.  The best list keeps KC >= k + 16
 // entries so that rounding in the expanded form cannot push a true neighbour
 // out of it.
@@ -650,7 +650,8 @@ __global__ void knn_emit_kernel(int64_t nq, const unsigned long long *__restrict
 // TMA ring) that both row blocks share.  Shared memory holds the operands
 // K-major in 128-byte-swizzled atoms (8 rows x 64 bfloat16).  Warp 9 allocates
 // the 512 TMEM columns: for each row block two 128 x 128 float32 accumulators
-// (tiles alternate between them).  One lane of it issues tcgen05.mma (M = 128,
+// (tiles alternate between them).  The warp runs converged and an elected lane of it
+// issues tcgen05.mma (M = 128,
 // N = 128, K = 16 per instruction, both row blocks per K step) and commits to
 // mbarriers that free the smem stage and hand the accumulators to the epilogue.
 // Warp 8 lane 0 issues the TMA loads.
@@ -661,8 +662,7 @@ __global__ void knn_emit_kernel(int64_t nq, const unsigned long long *__restrict
 // passes the threshold of any of the warp's rows appends their hits (tc_chunk) to the
 // rows' candidate buffers.  A row whose
 // buffer may not absorb another tile is merged into its sorted best list by its
-// warp: the buffer is sorted (bitonic, in registers) and a half-cleaner against
-// the reversed best list plus a bitonic merge keep the KC smallest.  No barrier
+// warp (merge_row).  No barrier
 // couples the epilogue warps: each arrives on the accumulator's "empty" barrier
 // when its TMEM reads are done and merges afterwards.  Every mbarrier wait gives
 // up after 2 s, records an error code and lets all roles reach the teardown,

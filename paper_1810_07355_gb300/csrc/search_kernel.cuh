@@ -28,8 +28,8 @@
 //   - the result set R, in registers, as a sorted list of at most k keys.
 // The up-to-e_s neighbours of the expanded node are tested and the new ones'
 // vectors gathered together: their ids go to shared gather slots in lane order, a
-// half warp reads each vector (several in flight per lane) and one transposed
-// // butterfly reduction for all of them).  R then takes the k
+// half warp reads each vector (several in flight per lane; at d > 256 the whole warp)
+// and one transposed butterfly reduction serves a round.  R then takes the k
 // best of R and the batch, and S takes the batch members within the new
 // r(1+eps).  Applying a batch at once yields the same R, the same r after the
 // batch and, since S only loses entries that can never be expanded, the same

@@ -572,7 +572,7 @@ def main():
     roof = {"bound": "hbm", "achieved": round(byt[head] / kern[head] / 1e9, 1), "peak": peak, "unit": "GB/s",
             "frac": round(byt[head] / kern[head] / 1e9 / peak, 4), "traffic": traffic,
             "kernel": f"search_kernel ({NAMES[head]})",
-            "peak_source": "measured hbm_gbs (burst), MEASURED_PEAKS.json",
+            "peak_source": "measured hbm_gbs (burst), MEASURED_PEAKS.json" if "hbm_gbs" in peaks else "6.8 TB/s",
             "frac_of_nominal_8tbs": round(byt[head] / kern[head] / 8e12, 4),
             "per_form": {f: {"achieved_gbs": round(byt[f] / kern[f] / 1e9, 1),
                              "frac": round(byt[f] / kern[f] / 1e9 / peak, 4),

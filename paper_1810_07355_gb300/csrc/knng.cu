@@ -848,48 +848,59 @@ __device__ __forceinline__ void tmem_wait32(uint32_t (&v)[32])
 enum { EPI_BYTE, EPI_FOLD, EPI_NORMS };
 
 // One 32-column chunk of a row: f[j] is column cb + j.  The maxima of eight groups of
-// four columns decide which groups any row of the warp needs; their hits are appended
-// from registers (static indices: a group is four predicated appends).  At 1M x 128
-// bytes, k = 100, two thirds of the chunks hold a hit of some row, and the branches over
-// the groups set the pace (about 20 cycles each): tested by halves first, most chunks
-// branch six times instead of eight, 277 -> 263 ms.  Reading hit columns back from TMEM
-// one by one is slower by a twentieth; four groups of eight columns take 267 ms, sixteen
-// of two 317, a jump by group number or anything else that writes f twice as long (the
-// next chunk's TMEM load then no longer runs ahead).
+// four columns give each row the groups that hold hits of its own; every row then takes
+// its next group at the same time, picking the group's four values out of its registers
+// by selects on the bits of the group number, and appends the hits among them.  At 1M x
+// 128 bytes, k = 100, two thirds of the chunks hold a hit of some row (1.3 on average),
+// so one turn mostly serves all rows, and a turn is 28 selects instead of branches over
+// the groups (about 20 cycles each): 277 ms with a branch for every group that any row
+// needs, 263 with these by halves, 240 as it is (252 without the vote on the chunk's
+// maximum; groups of two or eight columns 245, 255).  Reading hit columns back from TMEM
+// one by one is slower by a twentieth than the branches; a jump by group number, or
+// anything that writes f, takes twice as long (the next chunk's TMEM load then no longer
+// runs ahead).
 // sj = the row's own column in the chunk (self-joins), nl = columns of the chunk below n,
 // odd = the parity bits (EPI_BYTE).
 template <int EPI>
 __device__ __forceinline__ void tc_chunk(const float (&f)[32], float tr, float qnr, int cb, int sj, int nl, unsigned odd,
                                          unsigned long long *__restrict__ brow, int &cnt)
 {
-    float m[8];
+    constexpr int NG = 8;
+    float m[NG];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < NG; ++i)
         m[i] = fmaxf(fmaxf(f[i], f[i + 8]), fmaxf(f[i + 16], f[i + 24]));
     const float mx = fmaxf(fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])), fmaxf(fmaxf(m[4], m[5]), fmaxf(m[6], m[7])));
     if (!__any_sync(0xffffffffu, EPI == EPI_BYTE ? mx >= tr : mx > tr))
         return;
-    unsigned groups = 0;
+    unsigned groups = 0;  // this row's
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < NG; ++i)
         groups |= ((EPI == EPI_BYTE ? m[i] >= tr : m[i] > tr) ? 1u : 0u) << i;
-    groups = __reduce_or_sync(0xffffffffu, groups);
+#pragma unroll 1
+    do {
+        const bool any = groups != 0;
+        const int g = any ? __ffs((int)groups) - 1 : 0;
+        groups &= groups - 1;
 #pragma unroll
-    for (int h = 0; h < 8; h += 4) {
-        if (!(groups >> h & 15u))
-            continue;
+        for (int t = 0; t < 32; t += NG) {
+            float x[NG];
 #pragma unroll
-        for (int i = h; i < h + 4; ++i) {
-            if (!(groups >> i & 1u))
-                continue;
+            for (int i = 0; i < NG; ++i)
+                x[i] = f[t + i];
 #pragma unroll
-            for (int j = i; j < 32; j += 8) {
-                const float a = EPI == EPI_BYTE && (odd >> j & 1u) ? f[j] - 0.5f : f[j];
-                if ((EPI == EPI_BYTE ? a >= tr : a > tr) && j != sj && j < nl)
-                    brow[cnt++] = pack_key(fmaxf(qnr - 2.f * a, 0.f), cb + j);
+            for (int b = 1; b < NG; b *= 2) {
+                const bool upper = (g & b) != 0;
+#pragma unroll
+                for (int i = 0; i < NG; i += 2 * b)
+                    x[i] = upper ? x[i + b] : x[i];
             }
+            const int j = t + g;
+            const float a = EPI == EPI_BYTE && (odd >> j & 1u) ? x[0] - 0.5f : x[0];
+            if (any && (EPI == EPI_BYTE ? a >= tr : a > tr) && j != sj && j < nl)
+                brow[cnt++] = pack_key(fmaxf(qnr - 2.f * a, 0.f), cb + j);
         }
-    }
+    } while (__any_sync(0xffffffffu, groups != 0));
 }
 
 // Which base tiles a CTA sweeps, in order: its u-th tile is (t0 + g + u G) mod

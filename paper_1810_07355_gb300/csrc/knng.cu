@@ -670,7 +670,7 @@ __global__ void knn_emit_kernel(int64_t nq, const unsigned long long *__restrict
 constexpr int TC_M = 128, TC_N = 128, TC_BUF = BUF;
 constexpr int TC_RB = 2;                    // 128-row blocks per CTA
 // Buffered keys that trigger a merge: with the last tile's hits they mostly still fit one
-// chunk of 64 (64: 281, 56: 277, 48: 281, 32: 295 ms at 1M x 128 bytes, k = 100).
+// chunk of 64 (64: 246, 56: 240, 48: 245, 40: 251 ms at 1M x 128 bytes, k = 100).
 constexpr int TC_EAGER = 56;
 constexpr int TC_ROWS = TC_M * TC_RB;       // query rows per CTA
 constexpr int TC_EPI = 256;                 // epilogue threads (8 warps), one per row

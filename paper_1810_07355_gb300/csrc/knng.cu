@@ -301,7 +301,7 @@ __device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, un
 // next slab's global loads are in flight during the arithmetic of the present one.
 // With fewer row blocks than the device holds, several CTAs share a block's base tiles
 // (Shares) and knn_merge_kernel merges their lists: 50 queries over 1M x 128 ran on
-// one CTA before, 147.5 ms; 1.02 ms now.
+// one CTA before, 147.5 ms; 0.85 ms now (1.02 with the merges as loops).
 template <int RM> struct TileSmem {
     float2 As[2][BK][16 * RM];
     float Bs[2][BK][BN + 4];
@@ -1395,8 +1395,8 @@ __global__ void split_rows_kernel(const float *__restrict__ M, int64_t rows, int
 //   integer below 2^23): its 8-bit fields times 2^16, 2^8 and 1, each exact in
 //   bfloat16; zeros elsewhere.  The MMA then accumulates q.x - floor(|x|^2 / 2) exactly.
 //   Padding d to whole K atoms takes byte rows of any d = 32 .. 128 here from the float32
-//   sweep (30,011 x 100, the whole build: 20.5 -> 9.3 ms); below 32 the ties of small
-//   integers would flood the lists.
+//   sweep (30,011 x 100, the whole build: 20.5 -> 9.3 ms by this alone, 5.8 now); below
+//   32 the ties of small integers would flood the lists.
 __global__ void prepare_rows_kernel(const float *__restrict__ M, int64_t rows, int d, int dpa, bool base,
                                     float *__restrict__ norm, __nv_bfloat16 *__restrict__ out, int *flag)
 {

@@ -305,6 +305,10 @@ __global__ void __launch_bounds__(kPivThreads, kPivMinCta)
             sm.best[i][lane] = l[0];
             sm.best[i][32 + lane] = l[1];
         }
+        // Rows of one chunk write the next tile's distances before any further barrier;
+        // longer ones pass the barrier of their next tile's first chunk first.
+        if (d4 <= kPivD / 4)
+            __syncthreads();
     }
     if (S > 1)
         cluster.sync();

@@ -1213,8 +1213,10 @@ template <int V, class T, int HV, int KR> struct Warp {
             update_bound();
         // S <- S + batch members within r(1+eps)
         pool_push(isnew && d2 <= bnd, key);
-        if (predict && key_d2(pf_key) > bnd)
-            pf_key = kMaxKey;  // a batch member that was not pushed after all
+        // a batch member that was not pushed after all is not in S (the same comparison as
+        // the push: no key is within a bound that is NaN, from a NaN eps or distance)
+        if (predict && !(key_d2(pf_key) <= bnd))
+            pf_key = kMaxKey;
         if (predict == 2 && pf_key != kMaxKey) {
             // the row bounds were loading during the updates above
             pf_id = graph_id(lane < nm ? a.col[nbeg + lane] : -1);

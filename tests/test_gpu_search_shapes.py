@@ -59,3 +59,64 @@ def test_everything_visited(n):
     _compare(X, Q, g, seeds, min(10, n), 0, np.inf, 0, 0)
     st = _compare(X, Q, g, seeds, min(10, n), 24, np.inf, 24, 0)
     assert (st[:, 3] == 0).all()
+
+
+def _algorithm1(g, X, q, k, e_s, eps, seeds):
+    """Algorithm 1 a batch at a time (the seeds, then a node's scanned neighbours), with
+    IEEE comparisons and a NaN distance ordered after every number (ties by id): ids and
+    distances of R, distance computations, expansions."""
+    def key(i):
+        d2 = float(((X[i] - q) ** 2).sum())
+        return (np.inf if np.isnan(d2) else d2, int(i), d2)
+    f2 = (1.0 + float(np.float32(eps))) ** 2
+    R, S, seen, r2, bound, ndc, nexp = [], [], set(), np.nan, np.inf, 0, 0
+    batch, rset = list(dict.fromkeys(seeds.tolist())), False
+    while True:
+        init = nexp == 0
+        new = [key(i) for i in batch if i not in seen]
+        seen.update(batch)
+        ndc += len(new)
+        for c in new:
+            if init or not rset or c[2] <= r2:
+                R = sorted(R + [c])[:k]
+                if not init and len(R) == k:
+                    rset, r2 = True, R[-1][2]
+        if rset:
+            bound = r2 * f2
+        S = sorted(S + [c for c in new if c[2] <= bound])
+        if not S or S[0][2] > bound:
+            return [c[1] for c in R], [np.sqrt(c[2]) for c in R], ndc, nexp
+        node, nexp = S.pop(0)[1], nexp + 1
+        batch = g[1][g[0][node]:g[0][node + 1]][:e_s].tolist()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("padded", [0, 20])
+@pytest.mark.parametrize("nan", ["eps", "rows"])
+def test_nan_bound(nan, padded, prec):
+    """A NaN eps of some queries, or NaN coordinates that reach the k-th result, make the
+    bound NaN in the middle of a search: nothing is pushed from then on, the candidates
+    left are expanded, and the other queries are as ever."""
+    from paper_1810_07355_gb300 import onng
+    rng = np.random.default_rng(5)
+    X = synth.small_integers(600, 8, high=9, seed=1)
+    Q = synth.small_integers(24, 8, high=9, seed=2)
+    nbr, ln = oracle.knng(X, 30)
+    g = oracle.adjust_degree(nbr, ln, 12, 30)
+    seeds = rng.integers(0, 600, size=(24, 6)).astype(np.int32)
+    eps = np.full(24, 0.1, np.float32)
+    if nan == "eps":
+        eps[::3] = np.nan
+    else:
+        X[rng.integers(0, 600, size=200), 3] = np.nan
+    idx = onng.Index(_dev(g[0].astype(np.int64)), _dev(g[1].astype(np.int32)), _dev(X))
+    if padded:
+        idx.with_adjacency(padded)
+    ids, dist, st = onng.search(idx, _dev(Q), 10, 20, 0.1, _dev(seeds), eps_q=_dev(eps), precision=prec, k_rerank=10)
+    ids, dist, st = ids.cpu().numpy(), dist.cpu().numpy(), st.cpu().numpy()
+    for r in range(24):
+        o_ids, o_dist, ndc, nexp = _algorithm1(g, X, Q[r], 10, 20, eps[r], seeds[r])
+        m = len(o_ids)
+        assert np.array_equal(ids[r, :m], o_ids) and (ids[r, m:] == -1).all()
+        assert np.allclose(dist[r, :m], o_dist, rtol=1e-6, equal_nan=True)
+        assert tuple(st[r, :2]) == (ndc, nexp)

@@ -683,6 +683,7 @@ template <int V, class T, int HV, int KR> struct Warp {
             log_bits(isnew, id);
             return isnew;
         }
+        __syncwarp();  // every lane's `used` and tags are from before the batch
         unsigned short *half = reinterpret_cast<unsigned short *>(sm.vis);
         const unsigned used = p.x & 0xFFFFu;
         unsigned pos = 0;
@@ -744,6 +745,7 @@ template <int V, class T, int HV, int KR> struct Warp {
             return isnew;
         }
         const unsigned wm = __ballot_sync(FULL, want);
+        __syncwarp();  // the buckets are read before any is written; a batch always orders shared memory
         if (!wm)
             return false;
         const int used1 = (p0.x != -1) + (p0.y != -1) + (p0.z != -1) + (p0.w != -1) + (p1.x != -1) +
@@ -1045,6 +1047,7 @@ template <int V, class T, int HV, int KR> struct Warp {
     {
         if (no == 0 && ng == 0)
             return;
+        __syncwarp();  // keys that other lanes appended to the levels
         const Levels r = refill_slow<kOvf>({no, ng, 0, 0u, sm.tau, kMaxKey}, sm.ovf, gpool(), bnd, lane);
         no = r.no;
         ng = r.ng;

@@ -61,6 +61,20 @@ def test_everything_visited(n):
     assert (st[:, 3] == 0).all()
 
 
+@pytest.mark.parametrize("distinct", [1, 2, 5, 32])
+def test_repeated_seeds(distinct):
+    """Seeds that repeat few ids over a whole batch and over several: each counts once."""
+    X = synth.small_integers(400, 12, high=9, seed=3)
+    Q = synth.small_integers(16, 12, high=9, seed=4)
+    nbr, ln = oracle.knng(X, 20)
+    g = oracle.adjust_degree(nbr, ln, 10, 20)
+    rng = np.random.default_rng(distinct)
+    some = np.stack([rng.permutation(400)[:distinct] for _ in range(16)])
+    seeds = np.take_along_axis(some, rng.integers(0, distinct, size=(16, 64)), 1).astype(np.int32)
+    for padded in (0, 20):
+        _compare(X, Q, g, seeds, 10, 20, 0.1, padded, 0)
+
+
 def _algorithm1(g, X, q, k, e_s, eps, seeds):
     """Algorithm 1 a batch at a time (the seeds, then a node's scanned neighbours), with
     IEEE comparisons and a NaN distance ordered after every number (ties by id): ids and

@@ -71,6 +71,12 @@ int onng_version(void);
  * the expanded form |q|^2 + |x|^2 - 2 q.x, keep KC >= k + 16 survivors per row and
  * rescore them by direct difference in float32.  Inputs must be finite.
  *
+ * The workspace query does not fall as nq grows: a buffer for the largest batch
+ * serves every smaller one (n, d and k alike).  It asks for room to share the sweep of
+ * few queries among all SMs; a smaller buffer is planned into, down to about
+ * 2048 + 8 (k + 16 rounded up to a power of two, at least 32) bytes less for each of up
+ * to 58,368 spare lists, which leaves a list per query (two at d > 128).
+ *
  * onng_build_knng(X, n, d, k, ...) == onng_knn(X, n, d, X, n, k, 0, ...).
  */
 size_t onng_knn_workspace_bytes(int64_t n, int32_t d, int64_t nq, int32_t k);

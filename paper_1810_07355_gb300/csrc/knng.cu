@@ -249,30 +249,28 @@ __host__ __device__ __forceinline__ int64_t list_base(const Shares &sh, int g, i
     return ((int64_t)sh.gm * nq + (int64_t)(g - sh.gm) * tail - first) * per;
 }
 
-// lists (of one row each) that the shares of nq rows need
-int64_t list_rows(const Shares &sh, int64_t nq, int rows)
-{
-    const int64_t tail = sh.blocks > sh.main ? nq - sh.main * rows : 0;
-    return (int64_t)sh.gm * nq + (int64_t)(sh.gt - sh.gm) * tail;
-}
-
 // The shares of a sweep of `tiles` base tiles by `blocks` row blocks on `slots`
 // resident CTAs: whole waves unsplit (gm CTAs a block), and the blocks of the last,
 // partial wave split so that its CTAs end soonest (ceil(blocks gt / slots) rounds of
 // tiles / gt tiles, plus about `warm` tiles' worth for every further list: its
 // threshold starts from nothing).  200,000 x 100 floats, k = 100 (782 row blocks, 5.1
-// waves): the whole build 67.5 -> 64.2 ms.
-Shares plan_shares(int64_t blocks, int64_t tiles, int64_t slots, int gm, int64_t warm)
+// waves): the whole build 67.5 -> 64.2 ms.  Row blocks of `rows` queries; no more than
+// `lists` lists in all (at least gm nq).
+Shares plan_shares(int64_t nq, int64_t rows, int64_t tiles, int64_t slots, int gm, int64_t warm, int64_t lists)
 {
     Shares sh;
+    const int64_t blocks = (nq + rows - 1) / rows;
     sh.blocks = blocks;
     sh.gm = sh.gt = gm;
     sh.main = blocks * gm / slots * slots / gm;
     const int64_t rem = blocks - sh.main;
     if (rem == 0)
         return sh;
+    const int64_t tail = nq - sh.main * rows;
     int64_t best = INT64_MAX;
     for (int64_t g = gm; g <= std::min<int64_t>(std::max<int64_t>(tiles / 4, gm), std::max<int64_t>(8, slots / rem)); ++g) {
+        if (gm * nq + (g - gm) * tail > lists)
+            break;
         const int64_t cost = (rem * g + slots - 1) / slots * ((tiles + g - 1) / g + warm);
         if (cost < best) {
             best = cost;
@@ -1506,27 +1504,38 @@ int make_map(CUtensorMap *m, const void *ptr, int64_t rows, int d, int box_rows)
 // each, merged before the rescore.
 int split_share(int d) { return d > 128 ? 2 : 1; }
 
-// The plans of the two kinds of sweep.  They depend on the sizes alone, so the
-// workspace query and the call agree; kSweepSms is the GB300's SM count (two resident
-// CTAs per SM in the float32 sweep, one in the tensor-core sweeps).
-Shares plan_tile(int64_t n, int64_t nq, int rows)
-{
-    return plan_shares((nq + rows - 1) / rows, (n + BN - 1) / BN, 2 * kSweepSms, 1, 8);
-}
-
-Shares plan_tc(int64_t n, int d, int64_t nq, int kc)
-{
-    return plan_shares((nq + TC_ROWS - 1) / TC_ROWS, (n + TC_N - 1) / TC_N, kSweepSms, split_share(d), 8 * (int64_t)kc);
-}
-
 int tile_rows(int64_t nq) { return nq <= 16 ? 16 : nq <= 32 ? 32 : nq <= 64 ? 64 : 128; }
 
-// best lists (KC keys) and candidate buffers (BUF keys) a call needs, of one row each
-int64_t knn_list_rows(int64_t n, int d, int64_t nq, int kc)
+// Lists (of one row each: KC keys and a buffer of BUF) a call cannot do without, and
+// those its workspace request has room for.  The spare ones let every CTA that the
+// device holds keep lists of its own (a wave: two float32 CTAs of 128 rows, or one of 256
+// rows, per SM), as far as a sweep of n columns can be split that often; for some tens of
+// thousands of queries, whose row blocks fill about half a wave, two more for each (20,000
+// integer rows over 100,000 x 100: 28 ms with a wave's lists, 19 with these, 17 with six
+// more).  The request grows with nq, so a buffer for the largest batch serves every
+// smaller one; a smaller buffer is planned into (fewer shares).
+constexpr int64_t kWaveLists = 2 * kSweepSms * 128;
+static_assert(kWaveLists == (int64_t)kSweepSms * TC_ROWS, "a wave of either sweep holds as many rows");
+
+int64_t least_lists(int d, int64_t nq) { return nq * split_share(d); }
+
+int64_t asked_lists(int64_t n, int d, int64_t nq)
 {
-    const int rows = tile_rows(nq);
-    const int64_t a = list_rows(plan_tile(n, nq, rows), nq, rows);
-    return nq < TC_M ? a : std::max(a, list_rows(plan_tc(n, d, nq, kc), nq, TC_ROWS));
+    const int64_t most = std::max<int64_t>(1, std::min<int64_t>((n + BN - 1) / BN / 4, 2 * kSweepSms));
+    return least_lists(d, nq) + std::min(nq * (most - 1), std::max(kWaveLists, std::min(2 * nq, kWaveLists * 3 / 2)));
+}
+
+// The plans of the two kinds of sweep, for a workspace of `lists` lists.  kSweepSms is
+// the GB300's SM count (two resident CTAs per SM in the float32 sweep, one in the
+// tensor-core sweeps).
+Shares plan_tile(int64_t n, int64_t nq, int64_t lists)
+{
+    return plan_shares(nq, tile_rows(nq), (n + BN - 1) / BN, 2 * kSweepSms, 1, 8, lists);
+}
+
+Shares plan_tc(int64_t n, int d, int64_t nq, int kc, int64_t lists)
+{
+    return plan_shares(nq, TC_ROWS, (n + TC_N - 1) / TC_N, kSweepSms, split_share(d), 8 * (int64_t)kc, lists);
 }
 
 int pick_kc(int k)
@@ -1550,11 +1559,11 @@ int launch_tile(const float *X, int64_t n, int d, const float *Q, int64_t nq, in
 }
 
 template <int KC>
-int launch(const float *X, int64_t n, int d, const float *Q, int64_t nq, int k, int64_t self_offset, int32_t *nbr,
-           float *len, float *xn, float *qn, unsigned long long *best, unsigned long long *bufp, cudaStream_t s)
+int launch(const float *X, int64_t n, int d, const float *Q, int64_t nq, int k, const Shares &sh, int64_t self_offset,
+           int32_t *nbr, float *len, float *xn, float *qn, unsigned long long *best, unsigned long long *bufp,
+           cudaStream_t s)
 {
     const int rows = tile_rows(nq);
-    const Shares sh = plan_tile(n, nq, rows);
     int st = rows == 16   ? launch_tile<KC, 1>(X, n, d, Q, nq, self_offset, sh, xn, qn, best, bufp, s)
              : rows == 32 ? launch_tile<KC, 2>(X, n, d, Q, nq, self_offset, sh, xn, qn, best, bufp, s)
              : rows == 64 ? launch_tile<KC, 4>(X, n, d, Q, nq, self_offset, sh, xn, qn, best, bufp, s)
@@ -1580,13 +1589,12 @@ int launch_tc_kc(const CUtensorMap &ma, const CUtensorMap &mb, int64_t n, int64_
     return st ? st : merge_lists<KC>(sh, TC_ROWS, nq, best, s);
 }
 
-int launch_tc(const float *X, int64_t n, int d, const float *Q, int64_t nq, int k, int kc, int64_t self_offset,
-              int32_t *nbr, float *len, const float *xn, unsigned *par, float *qn, unsigned long long *best,
+int launch_tc(const float *X, int64_t n, int d, const float *Q, int64_t nq, int k, int kc, const Shares &sh,
+              int64_t self_offset, int32_t *nbr, float *len, const float *xn, unsigned *par, float *qn, unsigned long long *best,
               unsigned long long *bufp, int *err, __nv_bfloat16 *xb, __nv_bfloat16 *qb, cudaStream_t s)
 {
     const int gb = num_sms() * 8;
     const int dpa = (d + 63) / 64 * 64 + 64;  // whole K atoms; the extra one carries -floor(|x|^2 / 2)
-    const Shares sh = plan_tc(n, d, nq, kc);
     parity_kernel<<<gb, 256, 0, s>>>(xn, n, (n + TC_N - 1) / TC_N * (TC_N / 32), par);
     int st = check_launch("onng_knn: parity");
     if (st)
@@ -1632,8 +1640,8 @@ int launch_tcs_kc(const CUtensorMap *m, int64_t n, int64_t nq, int nk, const Sha
 
 // Float inputs on the tensor cores: centre, split into bfloat16 hi / lo, sweep
 // (knn_tcs_kernel), rescore the survivors from the original vectors.
-int launch_tcs(const float *X, int64_t n, int d, const float *Q, int64_t nq, int k, int kc, int64_t self_offset,
-               int32_t *nbr, float *len, float *xh, float *qn, unsigned long long *best, unsigned long long *bufp,
+int launch_tcs(const float *X, int64_t n, int d, const float *Q, int64_t nq, int k, int kc, const Shares &sh,
+               int64_t self_offset, int32_t *nbr, float *len, float *xh, float *qn, unsigned long long *best, unsigned long long *bufp,
                int *err, __nv_bfloat16 *xs, __nv_bfloat16 *qs, double *sums, float *mu, cudaStream_t s)
 {
     const int dp = (d + 63) / 64 * 64;
@@ -1654,7 +1662,6 @@ int launch_tcs(const float *X, int64_t n, int d, const float *Q, int64_t nq, int
         (st = make_map(&m[2], xhi, n, dp, TC_N)) || (st = make_map(&m[3], xlo, n, dp, TC_N)))
         return st;
     const int nk = dp / 64;
-    const Shares sh = plan_tc(n, d, nq, kc);
     auto sweep = [&](auto kcc) {
         constexpr int KC = decltype(kcc)::value;
         return fold ? launch_tcs_kc<KC, true>(m, n, nq, nk, sh, self_offset, xh, qn, best, bufp, err, s)
@@ -1680,6 +1687,40 @@ int launch_tcs(const float *X, int64_t n, int d, const float *Q, int64_t nq, int
     return check_launch("onng_knn: final kernel");
 }
 
+// The workspace of a call with room for `lists` lists; `used` is its size, which grows by
+// the same for every list (32-key lists are already whole 256-byte lines).
+struct KnnWs {
+    float *xn, *qn;
+    unsigned long long *best, *buf;
+    int *flags;
+    __nv_bfloat16 *xb, *qb;  // hi and lo rows of dp = 64 ceil(d / 64) (the byte path's rows of dp + 64 fit)
+    float *xh;
+    double *sums;
+    float *mu;
+    unsigned *par;
+    size_t used;
+
+    KnnWs(void *ws, int64_t n, int d, int64_t nq, int kc, int64_t lists)
+    {
+        n = std::max<int64_t>(n, 1);
+        nq = std::max<int64_t>(nq, 1);
+        const size_t dp = (size_t)(std::max(d, 1) + 63) / 64 * 64, tiles = (size_t)(n + TC_N - 1) / TC_N;
+        WsCarver c(ws);
+        xn = c.take<float>((size_t)n);
+        qn = c.take<float>((size_t)nq);
+        best = c.take<unsigned long long>((size_t)lists * kc);
+        buf = c.take<unsigned long long>((size_t)lists * BUF);
+        flags = c.take<int>(64);
+        xb = c.take<__nv_bfloat16>((size_t)n * dp * 2);
+        qb = c.take<__nv_bfloat16>((size_t)nq * dp * 2);
+        xh = c.take<float>(tiles * TC_N);
+        sums = c.take<double>((size_t)std::max(d, 1));
+        mu = c.take<float>((size_t)std::max(d, 1));
+        par = c.take<unsigned>(tiles * (TC_N / 32));
+        used = c.used;
+    }
+};
+
 }  // namespace
 }  // namespace onng
 
@@ -1687,23 +1728,8 @@ using namespace onng;
 
 extern "C" size_t onng_knn_workspace_bytes(int64_t n, int32_t d, int64_t nq, int32_t k)
 {
-    int kc = pick_kc(k);
-    WsCarver c(nullptr);
-    c.take<float>((size_t)std::max<int64_t>(n, 1));
-    c.take<float>((size_t)std::max<int64_t>(nq, 1));
-    const size_t lists = (size_t)knn_list_rows(std::max<int64_t>(n, 1), d, std::max<int64_t>(nq, 1), kc ? kc : 32);
-    c.take<unsigned long long>(lists * (kc ? kc : 32));
-    c.take<unsigned long long>(lists * BUF);
-    c.take<int>(64);
-    // bfloat16 copies: hi and lo rows of dp = 64 ceil(d / 64) (the byte path's rows of dp + 64 fit)
-    const size_t dp = (size_t)(std::max(d, 1) + 63) / 64 * 64;
-    c.take<__nv_bfloat16>((size_t)std::max<int64_t>(n, 1) * dp * 2);
-    c.take<__nv_bfloat16>((size_t)std::max<int64_t>(nq, 1) * dp * 2);
-    c.take<float>((size_t)(std::max<int64_t>(n, 1) + TC_N - 1) / TC_N * TC_N);
-    c.take<double>((size_t)std::max(d, 1));
-    c.take<float>((size_t)std::max(d, 1));
-    c.take<unsigned>((size_t)(std::max<int64_t>(n, 1) + TC_N - 1) / TC_N * (TC_N / 32));
-    return c.used;
+    const int kc = pick_kc(k) ? pick_kc(k) : 32;
+    return KnnWs(nullptr, n, d, nq, kc, asked_lists(std::max<int64_t>(n, 1), d, std::max<int64_t>(nq, 1))).used;
 }
 
 extern "C" int onng_knn(const float *X, int64_t n, int32_t d, const float *Q, int64_t nq, int32_t k,
@@ -1719,23 +1745,14 @@ extern "C" int onng_knn(const float *X, int64_t n, int32_t d, const float *Q, in
         return ONNG_OK;
     ONNG_REQUIRE(X && Q && nbr && len, ONNG_E_INVAL, "onng_knn: NULL pointer");
     ONNG_REQUIRE(aligned16(X) && aligned16(Q), ONNG_E_INVAL, "onng_knn: X and Q must be 16-byte aligned");
-    const size_t need = onng_knn_workspace_bytes(n, d, nq, k);
-    ONNG_REQUIRE(ws && ws_bytes >= need, ONNG_E_WORKSPACE, "onng_knn: workspace %zu < %zu bytes", ws_bytes, need);
     const int kc = pick_kc(k);
-    WsCarver c(ws);
-    float *xn = c.take<float>((size_t)std::max<int64_t>(n, 1));
-    float *qn = c.take<float>((size_t)nq);
-    const size_t lists = (size_t)knn_list_rows(std::max<int64_t>(n, 1), d, nq, kc);
-    unsigned long long *best = c.take<unsigned long long>(lists * kc);
-    unsigned long long *bufp = c.take<unsigned long long>(lists * BUF);
-    int *flags = c.take<int>(64);
-    const size_t dp = (size_t)(d + 63) / 64 * 64;
-    __nv_bfloat16 *xb = c.take<__nv_bfloat16>((size_t)std::max<int64_t>(n, 1) * dp * 2);
-    __nv_bfloat16 *qb = c.take<__nv_bfloat16>((size_t)nq * dp * 2);
-    float *xh = c.take<float>((size_t)(std::max<int64_t>(n, 1) + TC_N - 1) / TC_N * TC_N);
-    double *sums = c.take<double>((size_t)d);
-    float *mu = c.take<float>((size_t)d);
-    unsigned *par = c.take<unsigned>((size_t)(std::max<int64_t>(n, 1) + TC_N - 1) / TC_N * (TC_N / 32));
+    const size_t need = KnnWs(nullptr, n, d, nq, kc, least_lists(d, nq)).used;
+    ONNG_REQUIRE(ws && ws_bytes >= need, ONNG_E_WORKSPACE, "onng_knn: workspace %zu < %zu bytes", ws_bytes, need);
+    const int64_t lists = std::min(asked_lists(std::max<int64_t>(n, 1), d, nq),
+                                   least_lists(d, nq) + (int64_t)((ws_bytes - need) / ((kc + BUF) * sizeof(unsigned long long))));
+    const KnnWs w(ws, n, d, nq, kc, lists);
+    float *const xn = w.xn, *const qn = w.qn;
+    int *const flags = w.flags;
     cudaStream_t s = to_cuda(stream);
     // tensor-core paths (k + 16 <= 128, from one row block of queries): byte-valued inputs
     // at d = 32 .. 128 exactly; other non-integer inputs at d >= 32 by the split bfloat16
@@ -1747,8 +1764,8 @@ extern "C" int onng_knn(const float *X, int64_t n, int32_t d, const float *Q, in
         const int gb = num_sms() * 8;
         const bool byte_d = d >= 32 && d <= 128;
         const int dpa = (d + 63) / 64 * 64 + 64;
-        prepare_rows_kernel<<<gb, 256, 0, s>>>(Q, nq, d, dpa, false, qn, byte_d ? qb : nullptr, flags);
-        prepare_rows_kernel<<<gb, 256, 0, s>>>(X, n, d, dpa, true, xn, byte_d ? xb : nullptr, flags);
+        prepare_rows_kernel<<<gb, 256, 0, s>>>(Q, nq, d, dpa, false, qn, byte_d ? w.qb : nullptr, flags);
+        prepare_rows_kernel<<<gb, 256, 0, s>>>(X, n, d, dpa, true, xn, byte_d ? w.xb : nullptr, flags);
         st = check_launch("onng_knn: rows");
         if (st)
             return st;
@@ -1756,11 +1773,11 @@ extern "C" int onng_knn(const float *X, int64_t n, int32_t d, const float *Q, in
         ONNG_CUDA_TRY(cudaMemcpyAsync(&kind, flags, sizeof(int), cudaMemcpyDeviceToHost, s), "onng_knn: flag");
         ONNG_CUDA_TRY(cudaStreamSynchronize(s), "onng_knn: value check");
         if (!(kind & 1) && byte_d)
-            return launch_tc(X, n, d, Q, nq, k, kc, self_offset, nbr, len, xn, par, qn, best, bufp, flags + 1, xb,
-                             qb, s);
+            return launch_tc(X, n, d, Q, nq, k, kc, plan_tc(n, d, nq, kc, lists), self_offset, nbr, len, xn, w.par, qn,
+                             w.best, w.buf, flags + 1, w.xb, w.qb, s);
         if ((kind & 2) && d >= 32)
-            return launch_tcs(X, n, d, Q, nq, k, kc, self_offset, nbr, len, xh, qn, best, bufp, flags + 1, xb, qb,
-                              sums, mu, s);
+            return launch_tcs(X, n, d, Q, nq, k, kc, plan_tc(n, d, nq, kc, lists), self_offset, nbr, len, w.xh, qn, w.best,
+                              w.buf, flags + 1, w.xb, w.qb, w.sums, w.mu, s);
     } else {
         if (n > 0)
             norms_kernel<<<(unsigned)((n * 32 + 255) / 256), 256, 0, s>>>(X, n, d, xn);
@@ -1769,11 +1786,12 @@ extern "C" int onng_knn(const float *X, int64_t n, int32_t d, const float *Q, in
         if (st)
             return st;
     }
+    const Shares sh = plan_tile(n, nq, lists);
     switch (kc) {
-    case 32: return launch<32>(X, n, d, Q, nq, k, self_offset, nbr, len, xn, qn, best, bufp, s);
-    case 64: return launch<64>(X, n, d, Q, nq, k, self_offset, nbr, len, xn, qn, best, bufp, s);
-    case 128: return launch<128>(X, n, d, Q, nq, k, self_offset, nbr, len, xn, qn, best, bufp, s);
-    default: return launch<256>(X, n, d, Q, nq, k, self_offset, nbr, len, xn, qn, best, bufp, s);
+    case 32: return launch<32>(X, n, d, Q, nq, k, sh, self_offset, nbr, len, xn, qn, w.best, w.buf, s);
+    case 64: return launch<64>(X, n, d, Q, nq, k, sh, self_offset, nbr, len, xn, qn, w.best, w.buf, s);
+    case 128: return launch<128>(X, n, d, Q, nq, k, sh, self_offset, nbr, len, xn, qn, w.best, w.buf, s);
+    default: return launch<256>(X, n, d, Q, nq, k, sh, self_offset, nbr, len, xn, qn, w.best, w.buf, s);
     }
 }
 

@@ -40,6 +40,21 @@ def test_binding_covers_header():
     assert set(onng.exported_symbols()) <= _declared()
 
 
+@pytest.mark.parametrize("d,k", [(16, 1), (100, 100), (128, 10), (256, 100), (960, 200)])
+@pytest.mark.parametrize("n", [50, 3000, 100_000, 1_000_000])
+def test_knn_workspace_grows_with_the_batch(lib, n, d, k):
+    """A buffer sized for a batch serves every smaller one, and the room for sharing the
+    sweep (lists beyond one per query and share) stays bounded."""
+    sizes = [1, 2, 15, 16, 17, 32, 33, 64, 65, 127, 128, 129, 255, 256, 257, 511, 513, 1000, 5000, 9729, 10_000, 19_457,
+             20_000, 29_184, 29_185, 38_912, 38_913, 40_000, 77_825, 150_000, n]
+    need = [lib.onng_knn_workspace_bytes(n, d, nq, k) for nq in sorted(sizes)]
+    assert need == sorted(need)
+    kc = next(c for c in (32, 64, 128, 256) if k + 16 <= c)
+    per = 8 * (kc + 256) * (2 if d > 128 else 1) + 4 + 256 * ((d + 63) // 64)  # lists, norm and copies of a query
+    for nq, b in zip(sorted(sizes), need):
+        assert b <= need[0] + (nq - 1) * per + 58_368 * 8 * (kc + 256) + 4096
+
+
 def test_version_and_argument_checks(lib):
     from paper_1810_07355_gb300 import onng
     assert lib.onng_version() >= 1

@@ -54,3 +54,42 @@ def test_split_sweep_floats(nq, n, d):
     assert np.allclose(dist, o_dist, rtol=1e-5, atol=0)
     exact = np.sqrt(((X[ids].astype(np.float64) - Q[:, None].astype(np.float64)) ** 2).sum(2))
     assert np.allclose(dist, exact, rtol=1e-5, atol=0)
+
+
+@pytest.mark.parametrize("kind,n,d,nq,k", [("int", 6007, 36, 50, 10), ("int", 6007, 256, 300, 100), ("byte", 20_000, 100, 300, 100),
+                                           ("byte", 20_000, 128, 257, 10), ("float", 9000, 100, 300, 40),
+                                           ("float", 9000, 260, 257, 10), ("int", 3000, 16, 700, 200)])
+def test_workspace_sizes(kind, n, d, nq, k):
+    """Any workspace from one list per query and share up to the request (and beyond)
+    gives the same lists and is not overrun; a smaller one is refused."""
+    import torch
+
+    from paper_1810_07355_gb300 import onng
+    rng = np.random.default_rng(n + d)
+    if kind == "float":
+        X = rng.normal(size=(n + nq, d)).astype(np.float32)
+    else:
+        X = rng.integers(0, 256 if kind == "byte" else 300, size=(n + nq, d)).astype(np.float32)
+    X, Q = X[:n], X[n:]
+    o_ids, o_dist = oracle.knn(X, Q, k)
+    lib = onng.load()
+    kc, share, dp, tiles = next(c for c in (32, 64, 128, 256) if k + 16 <= c), 2 if d > 128 else 1, (d + 63) // 64 * 64, -(-n // 128)
+    least = 0
+    for b in (4 * n, 4 * nq, nq * share * kc * 8, nq * share * 256 * 8, 256, n * dp * 4, nq * dp * 4, tiles * 512, 8 * d, 4 * d,
+              tiles * 16):
+        least = -(-least // 256) * 256 + b
+    ask = lib.onng_knn_workspace_bytes(n, d, nq, k)
+    assert least <= ask
+    dX, dQ = torch.from_numpy(X).cuda(), torch.from_numpy(Q).cuda()
+    for size in (least, (2 * least + ask) // 3, ask - 1, ask, 2 * ask, least - 1):
+        ws = torch.full((size + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+        ids = torch.empty((nq, k), dtype=torch.int32, device="cuda")
+        dist = torch.empty((nq, k), device="cuda")
+        st = lib.onng_knn(onng._ptr(dX), n, d, onng._ptr(dQ), nq, k, -1, onng._ptr(ids), onng._ptr(dist), onng._ptr(ws), size,
+                          onng._stream())
+        assert st == (onng.ONNG_E_WORKSPACE if size < least else onng.ONNG_OK)
+        assert (ws[size:] == 0xA5).all()
+        if st == onng.ONNG_OK:
+            if kind != "float":
+                assert np.array_equal(ids.cpu().numpy(), o_ids)
+            assert np.allclose(dist.cpu().numpy(), o_dist, rtol=1e-5, atol=0)

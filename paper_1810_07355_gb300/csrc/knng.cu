@@ -151,7 +151,7 @@ template <int JL> __device__ __forceinline__ void pair_steps(unsigned long long 
 }
 
 // The warp merges row gr's cnt buffered keys into its sorted best list of KC
-// keys and returns the new threshold: the distance of list entry kth (< KC).
+// keys and returns list entry kth (< KC), whose distance is the new threshold.
 //
 // A merge holds up its whole CTA (the next tile's accumulators stay taken), so its
 // latency counts: element 64 h + 2 lane + r of the list sits in register m[h][r] of
@@ -163,8 +163,8 @@ template <int JL> __device__ __forceinline__ void pair_steps(unsigned long long 
 // against loops over the steps with element 32 r + lane (9,800 cycles a merge, now 5,900
 // with eight warps at it).
 template <int KC>
-__device__ __noinline__ float merge_row(int64_t gr, int cnt, int kth, unsigned long long *__restrict__ best,
-                                           const unsigned long long *__restrict__ buf, int lane)
+__device__ __noinline__ unsigned long long merge_row(int64_t gr, int cnt, int kth, unsigned long long *__restrict__ best,
+                                                     const unsigned long long *__restrict__ buf, int lane)
 {
     static_assert(BUF % 64 == 0 && (KC & (KC - 1)) == 0, "whole chunks and a power-of-two list");
     constexpr int H = KC < 64 ? 1 : KC / 64;
@@ -212,7 +212,7 @@ __device__ __noinline__ float merge_row(int64_t gr, int cnt, int kth, unsigned l
         if (kth >> 6 == h)
             kv = kth & 1 ? m[h][1] : m[h][0];
     }
-    return key_dist(__shfl_sync(0xffffffffu, kv, (kth >> 1) & 31));
+    return __shfl_sync(0xffffffffu, kv, (kth >> 1) & 31);
 }
 
 // Which share of a sweep a CTA takes.  The row blocks below `main` are swept by gm
@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(NT, 2)
                 break;
             const int c = s_cnt[r];
             if (c > BUF - BN || (last_tile && c > 0)) {
-                const float t = merge_row<KC>(grow, c, KC - 1, best, buf, lane);
+                const float t = key_dist(merge_row<KC>(grow, c, KC - 1, best, buf, lane));
                 if (lane == 0) {
                     s_thr[r] = t;
                     s_cnt[r] = 0;
@@ -839,7 +839,11 @@ __device__ __forceinline__ void tmem_wait32(uint32_t (&v)[32])
 //              corrected by the parity of |x|^2 (one bit per column) to a = q.x - |x|^2 / 2
 //              and kept when a >= tr, i.e. d^2 <= thr.  The comparison is not strict
 //              because thr is the k-th distance so far here (ranking is exact, so the list
-//              needs no slack): a later column at that distance may still win its tie by id.
+//              needs no slack): a later column at that distance may still win its tie by
+//              id.  In a tile whose ids all lie above the k-th entry's none can, and tr is
+//              raised by 1/2 (values are multiples of it), which leaves out the ties:
+//              100,000 equal rows of 36 bytes, k = 10, ran 162 ms with every tie appended
+//              and merged (39 on the float32 sweep).
 //   EPI_FOLD:  v = q.x - |x|^2 / 2 of the split form, the half norm added by spare columns
 //              of K; kept when v > tr.
 //   EPI_NORMS: v = q.x of the split form; the epilogue subtracts the half norms.
@@ -931,7 +935,7 @@ __device__ void tc_epilogue(uint64_t *accf, uint64_t *acce, uint32_t tmem, int w
     const float qnr = row_ok ? qn[grow] : 0.f;
     const int64_t self = (self_offset >= 0 && row_ok) ? self_offset + grow : -1;
     float thr = row_ok ? INFINITY : -INFINITY;
-    int cnt = 0;
+    int cnt = 0, kid = -1;  // kid: id of the list entry at thr
     unsigned long long *brow = buf + (row_ok ? grow : 0) * TC_BUF;
     const uint32_t lane_base = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(rb * 2 * TC_N);
     for (int64_t t = 0; t < tm.count; ++t) {
@@ -947,7 +951,9 @@ __device__ void tc_epilogue(uint64_t *accf, uint64_t *acce, uint32_t tmem, int w
         // d^2 = |q|^2 + |x|^2 - 2 q.x < thr  <=>  q.x - |x|^2 / 2 > (|q|^2 - thr) / 2, every
         // term an exact integer or half-integer for byte-valued inputs (approximate in
         // the split float form, whose survivors are rescored)
-        const float tr = 0.5f * (qnr - thr);
+        float tr = 0.5f * (qnr - thr);
+        if (EPI == EPI_BYTE && (int)col0 > kid)
+            tr += 0.5f;
         // columns of the tile below n (fewer than 128 in the last; none for rows that are no
         // query, whose accumulators may never have been written)
         const int cb0 = (int)col0, left = row_ok ? (int)min(n - col0, (int64_t)TC_N) : 0;
@@ -1003,9 +1009,10 @@ __device__ void tc_epilogue(uint64_t *accf, uint64_t *acce, uint32_t tmem, int w
             need &= need - 1;
             const int64_t gr = __shfl_sync(0xffffffffu, grow, src);
             const int c = __shfl_sync(0xffffffffu, cnt, src);
-            const float nt = merge_row<KC>(gr, c, kth, best, buf, lane);
+            const unsigned long long kk = merge_row<KC>(gr, c, kth, best, buf, lane);
             if (lane == src) {
-                thr = nt;
+                thr = key_dist(kk);
+                kid = key_id(kk);
                 cnt = 0;
             }
         }

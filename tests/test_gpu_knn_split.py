@@ -42,6 +42,23 @@ def test_byte_rows_any_dimension(n, d):
     assert np.allclose(dist, o_dist, rtol=1e-6, atol=0)
 
 
+@pytest.mark.parametrize("n,d,k,low", [(4000, 32, 10, 1), (4000, 36, 100, 1), (3000, 64, 40, 2), (5000, 128, 100, 2),
+                                       (2600, 68, 5, 0)])
+def test_byte_rows_all_tied(n, d, k, low):
+    """Rows whose k-th distance is shared by a large part of the base, or by all of it: the
+    smallest ids win, in sweeps that start at their own rows and wrap around, and in
+    those that several CTAs share."""
+    rng = np.random.default_rng(n)
+    X = np.full((n, d), 255, np.float32)
+    if low:
+        X[:, :low] = rng.integers(0, 2, size=(n, low))
+    for Q, o in ((X, 0), (X[::9].copy(), -1)):
+        ids, dist = _knn(X, Q, k, o)
+        o_ids, o_dist = oracle.knn(X, Q, k, np.arange(n) if o == 0 else None)
+        assert np.array_equal(ids, o_ids)
+        assert np.allclose(dist, o_dist, rtol=1e-6, atol=0)
+
+
 @pytest.mark.parametrize("nq,n,d", [(40, 5000, 100), (200, 5000, 100), (150, 3000, 260)])
 def test_split_sweep_floats(nq, n, d):
     """Float data: every position's length is the float64 one's to float32 rounding of

@@ -429,7 +429,11 @@ __device__ void path_row_warp(int64_t i, const int64_t *__restrict__ rp, const i
     __syncwarp();
     path_row_load(sm, beg, deg, col, len, lane, 32);
     __syncwarp();
-    const float lmax = sm.li[deg - 1];  // rows are sorted by length
+    // the longest edge, wherever it stands: a row that is nobody's neighbour need not be sorted
+    float lmax = 0.f;
+    for (int t = lane; t < deg; t += 32)
+        lmax = fmaxf(lmax, sm.li[t]);
+    lmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(lmax)));
     for (int u0 = 0; u0 < deg; u0 += 32)
         path_scan(sm, queue, beg, u0, deg, lmax, rp, col, len, lane);
     __syncwarp();

@@ -61,3 +61,37 @@ def test_degree_rows(n, k, e_o, e_i):
     want = oracle.adjust_degree(nbr, ln, e_o, e_i)
     for g, w in zip(got, want[:3]):
         assert np.array_equal(g.cpu().numpy(), w.astype(g.cpu().numpy().dtype))
+
+
+def test_row_order_of_nodes_without_in_edges():
+    """Only the rows of neighbours are searched by length: a node that nothing points to
+    may hold its edges (up to 256) in any order, or lengths that are no numbers behind
+    them, and loses the edges the rule says."""
+    import torch
+
+    from paper_1810_07355_gb300 import onng
+    rng = np.random.default_rng(8)
+    n, extra = 900, 60
+    X = rng.normal(size=(n + extra, 6)).astype(np.float32)
+    nbr, ln = oracle.knng(X[:n], 24)
+    ptr, col, length = oracle.adjust_degree(nbr, ln, 12, 24)
+    ptr, cols, lens = ptr.tolist(), [col], [length.astype(np.float32)]
+    for i in range(extra):
+        deg = [1, 2, 3, 31, 32, 33, 64, 100, 255, 256][i % 10]
+        d = np.sqrt(((X[:n] - X[n + i]) ** 2).sum(1))
+        c = np.argsort(d, kind="stable")[:deg]
+        l = d[c].astype(np.float32)
+        if i < 40:
+            o = rng.permutation(deg) if i < 30 else np.arange(deg)[::-1]
+            c, l = c[o], l[o]
+        else:
+            l[-max(1, deg // 8):] = np.nan
+        ptr.append(ptr[-1] + deg)
+        cols.append(c.astype(np.int32))
+        lens.append(l)
+    ptr, col, length = np.array(ptr, np.int64), np.concatenate(cols), np.concatenate(lens)
+    want = oracle.adjust_path(ptr, col, length, witnesses=True)
+    got = [t.cpu().numpy() for t in onng.adjust_path(*(torch.from_numpy(a).cuda() for a in (ptr, col, length)), witnesses=True)]
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+    assert np.array_equal(got[2], want[2].astype(np.float32), equal_nan=True)
+    assert np.array_equal(got[3], want[3])

@@ -252,12 +252,14 @@ __global__ void __launch_bounds__(kMlpWarps * 32)
     }
 }
 
-// Adam (Kingma & Ba 2015) on the flat vectors, step count t >= 1.
+// Adam (Kingma & Ba 2015) on the flat vectors, step count t >= 1.  The roundings are
+// written out (the decayed moment enters with a fused multiply-add), so that the one
+// step and the training run, which both call this, take the same ones.
 __device__ __forceinline__ void adam1(float &p, float g, float &m, float &v, float lr, float b1, float b2, float eps,
                                       float c1, float c2)
 {
-    m = b1 * m + (1.f - b1) * g;
-    v = b2 * v + (1.f - b2) * g * g;
+    m = fmaf(b1, m, __fmul_rn(1.f - b1, g));
+    v = fmaf(b2, v, __fmul_rn(__fmul_rn(1.f - b2, g), g));
     p -= lr * (m / c1) / (sqrtf(v / c2) + eps);
 }
 
@@ -573,12 +575,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
         for (int r = 0; r < kTrainPer; ++r) {
             const int e = tid + r * kTrainThreads;
             if (e < NP) {
-                // the fused forms adam1 compiles to where it was measured, written out: a
-                // rounding more or less would drift over the steps
-                const float g = s.G[e];
-                m[r] = fmaf(b1, m[r], (1.f - b1) * g);
-                v[r] = fmaf(b2, v[r], __fmul_rn((1.f - b2) * g, g));
-                p[r] -= lr * (m[r] / c1) / (sqrtf(v[r] / c2) + eps);
+                adam1(p[r], s.G[e], m[r], v[r], lr, b1, b2, eps, c1, c2);
                 train_store(s, e, p[r]);
             }
         }

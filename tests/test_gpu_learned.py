@@ -232,3 +232,27 @@ def test_learned_against_fixed_and_eq1_policies(onng):
     rho = spearmanr(host(y), host(eps_lab)).correlation
     print("held-out rank correlation of predicted and label eps:", round(float(rho), 3))
     assert np.isfinite(rho)
+
+
+def test_adam_roundings(onng):
+    """The moments after one step are m <- fl(b1 m + fl((1 - b1) g)) and
+    v <- fl(b2 v + fl(fl((1 - b2) g) g)), bit for bit (the outer sums in exact arithmetic)."""
+    from fractions import Fraction
+    rng = np.random.default_rng(11)
+    n = oracle.MLP_NPARAM
+    f = np.float32
+    P, G, M = (rng.normal(size=n).astype(f) for _ in range(3))
+    V = (rng.normal(size=n) ** 2).astype(f)
+    dP, dG, dM, dV = (torch.from_numpy(a.copy()).cuda() for a in (P, G, M, V))
+    onng.mlp_adam(dP, dG, dM, dV, 3, 1e-2)
+    b1, b2 = f(0.9), f(0.999)
+
+    def fused(b, x, t):  # b x + t rounded once
+        out = np.empty(n, f)
+        for i in range(n):
+            e = Fraction(float(b)) * Fraction(float(x[i])) + Fraction(float(t[i]))
+            c = f(float(e))  # within a rounding of it: the nearest of its neighbours is exact
+            out[i] = min((np.nextafter(c, f(-np.inf)), c, np.nextafter(c, f(np.inf))), key=lambda y: abs(Fraction(float(y)) - e))
+        return out
+    assert np.array_equal(dM.cpu().numpy(), fused(b1, M, (f(1) - b1) * G))
+    assert np.array_equal(dV.cpu().numpy(), fused(b2, V, (f(1) - b2) * G * G))

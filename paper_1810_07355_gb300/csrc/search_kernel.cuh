@@ -306,12 +306,6 @@ __device__ __forceinline__ u64 add_f32x2(u64 a, u64 b)
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
-__device__ __forceinline__ u64 mul_f32x2(u64 a, u64 b)
-{
-    u64 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 __device__ __forceinline__ u64 fma_f32x2(u64 a, u64 b, u64 c)
 {
     u64 r;
@@ -823,12 +817,17 @@ template <int V, class T, int HV, int KR> struct Warp {
             sa = fmaf(lo_f32(u1), lo_f32(u1), sa), sb = fmaf(lo_f32(u3), lo_f32(u3), sb);
             return pack_f32x2(fmaf(hi_f32(u1), hi_f32(u1), sa), fmaf(hi_f32(u3), hi_f32(u3), sb));
         } else {
-            u64 x[4] = {pack_f32x2(xa.x, xb.x), pack_f32x2(xa.y, xb.y), pack_f32x2(xa.z, xb.z), pack_f32x2(xa.w, xb.w)};
+            const float a4[4] = {xa.x, xa.y, xa.z, xa.w}, b4[4] = {xb.x, xb.y, xb.z, xb.w};
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
+                u64 x;
                 if constexpr (std::is_same<L, Loader<__nv_fp8_e4m3>>::value)
-                    x[c] = mul_f32x2(sp[v][c], x[c]);  // dequantised with a rounded product
-                const u64 u = add_f32x2(x[c], qp[v][c]);
+                    // dequantised with a rounded product (the packed multiply and the packed add
+                    // after it came out as one rounding)
+                    x = pack_f32x2(__fmul_rn(lo_f32(sp[v][c]), a4[c]), __fmul_rn(hi_f32(sp[v][c]), b4[c]));
+                else
+                    x = pack_f32x2(a4[c], b4[c]);
+                const u64 u = add_f32x2(x, qp[v][c]);
                 acc = fma_f32x2(u, u, acc);
             }
             return acc;

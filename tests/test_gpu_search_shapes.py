@@ -134,3 +134,26 @@ def test_nan_bound(nan, padded, prec):
         assert np.array_equal(ids[r, :m], o_ids) and (ids[r, m:] == -1).all()
         assert np.allclose(dist[r, :m], o_dist, rtol=1e-6, equal_nan=True)
         assert tuple(st[r, :2]) == (ndc, nexp)
+
+
+@pytest.mark.parametrize("d", [20, 128, 132, 256, 260, 516, 960])
+def test_fp8_products_are_rounded(d):
+    """A stored vector is the float32 product of scale and code: a query equal to it is at
+    distance 0 exactly (the probe's nearest-seed feature is the log of 1e-6)."""
+    import ctypes as C
+
+    from paper_1810_07355_gb300 import onng
+    rng = np.random.default_rng(d)
+    X = (100.0 * rng.random((300, d))).astype(np.float32)
+    Q = oracle.fp8_quantize(X)[2][:64]
+    idx = onng.Index(_dev(np.zeros(301, np.int64)), _dev(np.zeros(1, np.int32)), _dev(X)).with_fp8()
+    Qd, seeds = _dev(Q), _dev(np.stack([np.arange(64), np.arange(64) + 100], 1).astype(np.int32))
+    lib, p, ic = onng.load(), onng._Params(2, 0, 0.1, onng.PREC_FP8, 2, 1, 0), idx._c()
+    ws = torch.empty(lib.onng_search_workspace_bytes(64, C.byref(ic), C.byref(p)), dtype=torch.uint8, device="cuda")
+    feat = torch.empty((64, 16), device="cuda")
+    onng._check(lib.onng_search_probe(C.byref(ic), onng._ptr(Qd), 64, C.byref(p), onng._ptr(seeds), 2, 0.9, onng._ptr(feat), None,
+                                      onng._ptr(ws), ws.numel(), onng._stream()))
+    f = feat.cpu().numpy()
+    assert np.abs(f[:, 1] - np.log(1e-6)).max() < 1e-4
+    want = np.sqrt(((oracle.fp8_quantize(X)[2][100:164].astype(np.float64) - Q) ** 2).sum(1))
+    assert np.allclose(np.exp(f[:, 2]) * 1e-6, want, rtol=1e-4)

@@ -28,8 +28,7 @@
 //   - the result set R, in registers, as a sorted list of at most k keys.
 // The up-to-e_s neighbours of the expanded node are tested and the new ones'
 // vectors gathered together: their ids go to shared gather slots in lane order, a
-// half warp reads each vector (several in flight per lane; at d > 256 the whole warp)
-// and one transposed butterfly reduction serves a round.  R then takes the k
+// half warp reads each vector (several in flight per lane) and one transposed butterfly reduction serves a round.  R then takes the k
 // best of R and the batch, and S takes the batch members within the new
 // r(1+eps).  Applying a batch at once yields the same R, the same r after the
 // batch and, since S only loses entries that can never be expanded, the same
@@ -70,10 +69,12 @@
 #include "common.cuh"
 #include "warp_sort.cuh"
 
-// 1: float32: once the adjacency row of the node expanded next has arrived, ask L2 for
-// its neighbours' vectors (the next round's gathers then start from L2: 10,000 queries
-// on 1M x 128 4.8 ms without, 4.4 with).  The shorter vectors of the reduced forms are
-// better off without the extra instructions (bfloat16 2.95 ms with, 2.84 without).
+// 1: float32 at d <= 256: once the adjacency row of the node expanded next has arrived, ask
+// L2 for its neighbours' vectors (the next round's gathers then start from L2: 10,000
+// queries on 1M x 128 4.8 ms without, 4.4 with).  The shorter vectors of the reduced forms
+// are better off without the extra instructions (bfloat16 2.95 ms with, 2.84 without), and
+// so are longer ones, of which most neighbours' lines are not needed (100,000 x 960, 2,000
+// queries 7.8 ms with, 5.8 without).
 #ifndef ONNG_SEARCH_PREFETCH
 #define ONNG_SEARCH_PREFETCH 1
 #endif
@@ -557,11 +558,19 @@ template <int OVF> __device__ __noinline__ Levels refill_slow(Levels s, u64 *ovf
 // Every member is inlined: one call out of line would move the whole search state
 // from registers to local memory (the k > 32 kernels ran that way).
 template <int V, class T, int HV, int KR> struct Warp {
-    // d <= 256: a half warp reads each vector, so a lane holds two quads of it per
-    // 128 coordinates; above, the whole warp does (half the query registers)
-    static constexpr bool kHalf = V <= 2;
-    static constexpr int kPairs = V == 1 ? Tune<T>::pairs : 4;  // most vector pairs gathered per round by half warps
-    static constexpr int G = V >= 8 ? 2 : 4;  // vectors per gather round of the whole-warp form
+    // A half warp reads each vector, so a lane holds two quads of it per 128 coordinates;
+    // the whole warp does where the query, its scales and the lists leave no registers for
+    // that (FP8 above d = 512 with lists of more than 32).  d = 960, n = 100,000, ms with the
+    // whole warp and with halves: float32, one query 4.11, 1.98, 2,000 queries 12.9, 5.8;
+    // bfloat16 2.91, 2.46 and 8.45, 6.55; FP8 3.18, 2.72 and 8.15, 7.19, but 6.15, 7.19 with
+    // lists of 100.
+    static constexpr bool kHalf = V <= 4 || KR == 1 || !std::is_same<T, __nv_fp8_e4m3>::value;
+    static constexpr int G = 2;  // vectors per gather round of the whole-warp form
+    // Most vector pairs gathered per round by half warps, of stored vectors and of the
+    // float32 ones of a reduced form's rerank: a round's loads are in flight together, as
+    // far as registers go.
+    template <class L>
+    static constexpr int kPairs = V == 1 ? Tune<T>::pairs : V == 2 ? 4 : V == 8 && !std::is_same<L, Loader<T>>::value ? 1 : 2;
     static constexpr int kOvf = Tune<T>::ovf;  // shared-memory overflow keys
     static_assert(kOvf >= 64 && (kOvf & (kOvf - 1)) == 0, "the overflow holds a power of two >= 64 keys");
     static_assert(HV % 8 == 0, "the visited table holds whole buckets of 8 ids");
@@ -874,8 +883,10 @@ template <int V, class T, int HV, int KR> struct Warp {
                 acc = accumulate<L>(acc, raw[p][v][0], raw[p][v][1], v);
             s[p] = lo_f32(acc) + hi_f32(acc);
         }
-        tr_stage<PG, 8>(s, lane, PG);
-        tr_stage<PG, 4>(s, lane, PG / 2);
+        if constexpr (PG >= 2)
+            tr_stage<PG, 8>(s, lane, PG);
+        if constexpr (PG >= 4)
+            tr_stage<PG, 4>(s, lane, PG / 2);
         if constexpr (PG == 8)
             tr_stage<PG, 2>(s, lane, 2);
         float r = s[0];
@@ -905,14 +916,14 @@ template <int V, class T, int HV, int KR> struct Warp {
         __syncwarp();
         float mine = 0.0f;
         if constexpr (kHalf) {
-            constexpr int PG = std::is_same<L, Loader<float>>::value && V == 2 ? 4 : kPairs;
+            constexpr int PG = kPairs<L>, few = PG < 4 ? PG : 4;
             int b0 = 0;
             while (m - b0 > 8 && PG == 8) {
                 mine = gather_pairs<L, PG>(base, b0, m, rank, mine_in, mine);
                 b0 += 2 * PG;
             }
-            for (; b0 < m; b0 += 8)
-                mine = gather_pairs<L, 4>(base, b0, m, rank, mine_in, mine);
+            for (; b0 < m; b0 += 2 * few)
+                mine = gather_pairs<L, few>(base, b0, m, rank, mine_in, mine);
         } else {
             for (int b0 = 0; b0 < m; b0 += G) {
                 int gid[G];
@@ -1228,7 +1239,7 @@ template <int V, class T, int HV, int KR> struct Warp {
             }
         }
 #if ONNG_SEARCH_PREFETCH
-        if (sizeof(T) == 4 && predict && pf_key != kMaxKey && pf_id >= 0) {
+        if (sizeof(T) == 4 && V <= 2 && predict && pf_key != kMaxKey && pf_id >= 0) {
             // the row of the next node is in: its neighbours' vectors into L2
             const int bytes = a.d * (int)sizeof(T);  // float32 4, bfloat16 2, e4m3 1 byte per coordinate
             const char *row = static_cast<const char *>(xs) + (int64_t)pf_id * bytes;
@@ -1511,10 +1522,12 @@ template <int V, class T, int HV, int KR> struct Warp {
 };
 
 // Resident CTAs per SM the register budget is sized for.  Shared memory holds
-// 6 CTAs of warps with a 2048-slot table and 128 overflow keys (37 KB a CTA).
+// 6 CTAs of warps with a 2048-slot table and 128 overflow keys (37 KB a CTA).  Above d =
+// 256 a round's loads need more registers than three CTAs leave (100,000 x 960 float32,
+// 2,000 queries: 9.8 ms at 3, 7.8 at 2).
 template <class T> __host__ __device__ constexpr int min_blocks(int V, int KR)
 {
-    return V <= 2 && KR == 1 ? Tune<T>::minb : 3;
+    return V > 2 ? 2 : KR == 1 ? Tune<T>::minb : 3;
 }
 
 template <int V, class T, int HV, int KR>

@@ -46,6 +46,13 @@ def test_dimensions(d, prec):
     _compare(X, Q, g, seeds, 10, 20, 0.2, 20, prec, cap=5)
 
 
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("d", [384, 388, 448, 512, 576, 1020, 1024])
+def test_long_vectors(d, prec):
+    """The same where a lane holds up to sixteen quads of a vector, whole and partial."""
+    test_dimensions(d, prec)
+
+
 @pytest.mark.parametrize("n", [2, 513, 6000, 20000])
 def test_everything_visited(n):
     """eps = inf visits every node: from a table that stays nearly empty to one that

@@ -210,7 +210,9 @@ __global__ void __launch_bounds__(kPivThreads, kPivMinCta)
     };
     // arithmetic: warp -> 16 queries x 64 pivots, lane -> 4 queries x (4 + 4) pivots
     const int tq = (warp & 1) * 16 + (lane & 3) * 4, tp = (warp >> 1) * 64 + (lane >> 2) * 4;
-    const bool busy = (warp & 1) * 16 < nrow;
+    // (a warp whose queries or pivots are all padding skips the arithmetic: one query against
+    // 64 pivots at d = 1,024 took 108 us with every warp at it)
+    const int pivots = (warp & 1) * 16 < nrow ? te - (warp >> 1) * 64 : 0;  // busy in tiles from below this
     unsigned long long acc[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -230,7 +232,7 @@ __global__ void __launch_bounds__(kPivThreads, kPivMinCta)
             const int nt = last ? t0 + kPivT : t0, nc = last ? 0 : c0 + kPivD / 4;
             if (nt < te)
                 fetch(nt, nc);
-            if (busy) {
+            if (t0 < pivots) {
 #pragma unroll
                 for (int c = 0; c < kPivD; ++c) {
                     const ulonglong2 x0 = *reinterpret_cast<const ulonglong2 *>(&sm.ts[b][c][tp]);
@@ -348,6 +350,113 @@ __global__ void __launch_bounds__(kPivThreads, kPivMinCta)
         cluster.sync();  // no CTA leaves while another reads its lists
 }
 
+// The same rule for few pivots, where the tiles above are mostly padding and a chunk's
+// arithmetic does not cover the next one's loads: 16 queries x tiles of 64 pivots, chunks
+// of 64 coordinates, a thread per query and four pivots (16 apart), the same float32 chain
+// per pair.  A warp keeps the lists of two queries in registers.
+//
+// Taken for one tile, and for two where its blocks are fewer than the SMs but more than
+// one (few_pivots).  1,000 queries, us with the tiled kernel and with this one: 64 pivots
+// at d = 128 22 and 11, at d = 1,024 85 and 47; 100 pivots at d = 128 23 and 18, at d = 1,024 89
+// and 88; but 100 pivots at d = 128 for one query 14 and 18, for 10,000 49 and 58.
+constexpr int kFewQ = 16;
+constexpr int kFewT = 64;
+constexpr int kFewD = 64;
+
+__global__ void __launch_bounds__(kPivThreads, 5)
+    seeds_few_kernel(const float *__restrict__ X, int64_t n, int d, const float *__restrict__ Q, int64_t nq, int P, int n_seed,
+                     int32_t *__restrict__ out)
+{
+    __shared__ __align__(16) float qs[kFewQ][kFewD];
+    __shared__ __align__(16) float ts[kFewT][kFewD + 4];  // padded: 16 rows apart in distinct banks
+    __shared__ float dist[kFewQ][kFewT];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int qi = tid >> 4, pj = tid & 15;
+    const int64_t q0 = (int64_t)blockIdx.x * kFewQ;
+    const int d4 = d >> 2;
+    const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    unsigned long long best[2][2];  // queries warp and warp + 8 of the block
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+        best[i][0] = best[i][1] = kNoKey;
+    for (int t0 = 0; t0 < P; t0 += kFewT) {
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int c0 = 0; c0 < d4; c0 += kFewD / 4) {
+            __syncthreads();  // the chunk before has been read (and the tile before folded)
+            {
+                const int r = tid >> 4, c = c0 + (tid & 15);
+                reinterpret_cast<float4 *>(qs[r])[tid & 15] =
+                    q0 + r < nq && c < d4 ? __ldg(reinterpret_cast<const float4 *>(Q + (q0 + r) * d) + c) : zero4;
+            }
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                const int r = g * 16 + (tid >> 4), t = t0 + r, c = c0 + (tid & 15);
+                reinterpret_cast<float4 *>(ts[r])[tid & 15] =
+                    t < P && c < d4 ? __ldg(reinterpret_cast<const float4 *>(X + (int64_t)t * n / P * d) + c) : zero4;
+            }
+            __syncthreads();
+#pragma unroll 4
+            for (int c = 0; c < kFewD / 4; ++c) {
+                const float4 a = reinterpret_cast<const float4 *>(qs[qi])[c];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float4 b = reinterpret_cast<const float4 *>(ts[pj + 16 * j])[c];
+                    float u = b.x - a.x;
+                    acc[j] = fmaf(u, u, acc[j]);
+                    u = b.y - a.y;
+                    acc[j] = fmaf(u, u, acc[j]);
+                    u = b.z - a.z;
+                    acc[j] = fmaf(u, u, acc[j]);
+                    u = b.w - a.w;
+                    acc[j] = fmaf(u, u, acc[j]);
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            dist[qi][pj + 16 * j] = acc[j];
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            unsigned long long s[4] = {best[i][0], best[i][1], kNoKey, kNoKey};
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int t = t0 + 32 * h + lane;
+                const float dv = dist[warp + 8 * i][32 * h + lane];
+                if (t < P && !isnan(dv))
+                    s[2 + h] = pack_key(dv, t);
+            }
+            if (t0 == 0) {
+                best[i][0] = s[2];
+                best[i][1] = s[3];
+                warp_bitonic_sort<2>(best[i], lane);
+            } else {
+                warp_bitonic_sort<4>(s, lane);
+                best[i][0] = s[0];
+                best[i][1] = s[1];
+            }
+        }
+    }
+    const int m = n_seed < P ? n_seed : P;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int64_t q = q0 + warp + 8 * i;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = h * 32 + lane;
+            if (q < nq && r < n_seed)
+                out[q * n_seed + r] = r >= m || best[i][h] == kNoKey
+                                          ? -1
+                                          : (int32_t)((int64_t)(unsigned)(best[i][h] & 0xFFFFFFFFull) * n / P);
+        }
+    }
+}
+
+bool few_pivots(int64_t nq, int P)
+{
+    return P <= kFewT || (P <= 2 * kFewT && nq > kFewQ && nq <= (int64_t)kFewQ * num_sms());
+}
+
 // CTAs per cluster: how often the pivots of a query block are split.  The grid's time
 // is waves x (tiles per CTA + the fixed selection and merge work, about 64
 // coordinates' worth of a tile); the smallest split with the least such time is taken.
@@ -412,6 +521,11 @@ extern "C" int onng_seeds_pivot(const float *X, int64_t n, int32_t d, const floa
     ONNG_REQUIRE(X && Q && out, ONNG_E_INVAL, "onng_seeds_pivot: NULL pointer");
     ONNG_REQUIRE(aligned16(X) && aligned16(Q), ONNG_E_INVAL, "onng_seeds_pivot: X and Q must be 16-byte aligned");
     const int P = (int)std::min<int64_t>(n_pivot, n);
+    if (few_pivots(nq, P)) {
+        seeds_few_kernel<<<(unsigned)((nq + kFewQ - 1) / kFewQ), kPivThreads, 0, to_cuda(stream)>>>(X, n, d, Q, nq, P, n_seed,
+                                                                                                    out);
+        return check_launch("onng_seeds_pivot");
+    }
     const size_t sm = sizeof(PivSmem);
     ONNG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void *>(seeds_pivot_kernel),
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm),

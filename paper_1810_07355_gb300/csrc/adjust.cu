@@ -1173,12 +1173,17 @@ extern "C" int onng_adjust_path(const int64_t *row_ptr, const int32_t *col, cons
         const int64_t resident = (int64_t)num_sms() * std::max(per_sm, 1);
         const int64_t ctas = std::min<int64_t>((n + kPathWarps - 1) / kPathWarps, resident);
         path_small_kernel<<<(unsigned)ctas, kPathWarps * 32, 0, s>>>(row_ptr, col, len, n, wit, big, n_big);
-        // longer rows: the kernels read the counts of listed rows on the device
-        ONNG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void *>(path_long_kernel),
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PathLong)),
-                      "adjust_path: smem attribute");
-        path_mid_kernel<<<num_sms() * 8, 256, 0, s>>>(row_ptr, col, len, wit, big, n_big);
-        path_long_kernel<<<num_sms(), 1024, sizeof(PathLong), s>>>(row_ptr, col, len, n, wit, big, n_big);
+        // longer rows, of which nnz edges hold only so many: the kernels read the counts of
+        // listed rows on the device (two launches that find none cost a small graph 9 us)
+        if (nnz > kPathSmall)
+            path_mid_kernel<<<(unsigned)std::min<int64_t>(num_sms() * 8, nnz / (kPathSmall + 1)), 256, 0, s>>>(
+                row_ptr, col, len, wit, big, n_big);
+        if (nnz > kPathMid) {
+            ONNG_CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void *>(path_long_kernel),
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PathLong)),
+                          "adjust_path: smem attribute");
+            path_long_kernel<<<num_sms(), 1024, sizeof(PathLong), s>>>(row_ptr, col, len, n, wit, big, n_big);
+        }
         st = check_launch("onng_adjust_path: mark");
         if (st)
             return st;

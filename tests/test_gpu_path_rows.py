@@ -95,3 +95,41 @@ def test_row_order_of_nodes_without_in_edges():
     assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
     assert np.array_equal(got[2], want[2].astype(np.float32), equal_nan=True)
     assert np.array_equal(got[3], want[3])
+
+
+@pytest.mark.parametrize("n,deg", [(1, 0), (40, 1), (50, 5), (51, 5), (300, 257), (1100, 1025)])
+def test_few_edges_and_workspace_bounds(n, deg):
+    """Graphs too small to hold a row of the next size, and those just large enough; the
+    call stays within a workspace of exactly the requested size."""
+    import ctypes as C
+
+    import torch
+
+    from paper_1810_07355_gb300 import onng
+    rng = np.random.default_rng(n)
+    rp = np.minimum(np.arange(n + 1) * deg, deg * (n if n < 100 else 5)).astype(np.int64)
+    nnz = int(rp[-1])
+    col, ln = np.empty(nnz, np.int32), np.empty(nnz, np.float32)
+    for i in range(n):
+        m = int(rp[i + 1] - rp[i])
+        ids = rng.choice(n - 1, m, replace=False) if m else np.empty(0, np.int64)
+        ids = np.where(ids >= i, ids + 1, ids)
+        length = rng.integers(1, 20, size=m).astype(np.float32)
+        o = np.lexsort((ids, length))
+        col[rp[i]:rp[i + 1]], ln[rp[i]:rp[i + 1]] = ids[o], length[o]
+    want = oracle.adjust_path(rp, col, ln, witnesses=True)
+    lib = onng.load()
+    size = lib.onng_adjust_path_workspace_bytes(n, nnz)
+    ws = torch.full((size + 4096,), 0xA5, dtype=torch.uint8, device="cuda")
+    d_rp, d_col, d_ln = (torch.from_numpy(v).cuda() for v in (rp, np.append(col, 0).astype(np.int32), np.append(ln, 0).astype(np.float32)))
+    o_rp = torch.empty(n + 1, dtype=torch.int64, device="cuda")
+    o_col, o_wit = (torch.full((nnz + 1,), -7, dtype=torch.int32, device="cuda") for _ in range(2))
+    o_ln = torch.empty(nnz + 1, device="cuda")
+    kept = C.c_int64(0)
+    onng._check(lib.onng_adjust_path(onng._ptr(d_rp), onng._ptr(d_col), onng._ptr(d_ln), n, onng._ptr(o_rp), onng._ptr(o_col),
+                                     onng._ptr(o_ln), C.byref(kept), onng._ptr(o_wit), onng._ptr(ws), size, onng._stream()))
+    assert (ws[size:] == 0xA5).all()
+    m = kept.value
+    assert np.array_equal(o_rp.cpu().numpy(), want[0]) and m == len(want[1])
+    assert np.array_equal(o_col[:m].cpu().numpy(), want[1]) and np.array_equal(o_ln[:m].cpu().numpy(), want[2].astype(np.float32))
+    assert np.array_equal(o_wit[:nnz].cpu().numpy(), want[3])

@@ -1137,7 +1137,6 @@ extern "C" size_t onng_adjust_path_workspace_bytes(int64_t n, int64_t nnz)
     c.take<int64_t>((size_t)std::max<int64_t>(n, 1));      // kept counts / long rows
     c.take<int64_t>((size_t)std::max<int64_t>(n, 1));
     c.take<int>(64);
-    c.take<unsigned long long>(4);
     c.take<char>(scan_workspace_bytes(std::max<int64_t>(n, 1)));
     return c.used;
 }
@@ -1162,7 +1161,6 @@ extern "C" int onng_adjust_path(const int64_t *row_ptr, const int32_t *col, cons
     int64_t *kept = c.take<int64_t>((size_t)std::max<int64_t>(n, 1));
     int64_t *big = c.take<int64_t>((size_t)std::max<int64_t>(n, 1));
     int *n_big = c.take<int>(64);
-    c.take<unsigned long long>(4);
     char *scan_ws = c.take<char>(scan_workspace_bytes(std::max<int64_t>(n, 1)));
     int st;
     if (n > 0) {

@@ -68,6 +68,42 @@ def test_everything_visited(n):
     assert (st[:, 3] == 0).all()
 
 
+@pytest.mark.parametrize("n", [(1 << 23) - 1, 1 << 23, (1 << 23) + 1])
+def test_visited_set_at_the_widest_tags_and_beyond(n):
+    """The last size whose ids fit a bucket number and 14 tag bits, and the table of ids
+    above it: 12,000 linked nodes spread over the ids up to n - 1, rows of more than 32
+    entries, repeated seeds, few and all nodes visited (the tables and then the bitmap),
+    several queries per warp of a single CTA's workspace."""
+    from paper_1810_07355_gb300 import onng
+    rng = np.random.default_rng(n % 1000)
+    some = np.unique(np.concatenate([rng.integers(0, n, size=12_000), [0, 1, n // 2, n - 2, n - 1]])).astype(np.int32)
+    m = len(some)
+    deg = np.zeros(n, np.int64)
+    deg[some] = np.where(np.arange(m) % 50 == 0, 75, 25)
+    ptr = np.concatenate([[0], np.cumsum(deg)])
+    col = np.concatenate([some[rng.choice(m, deg[i], replace=False)] for i in some])
+    X = np.zeros((n, 4), np.float32)
+    X[some] = rng.integers(0, 64, size=(m, 4))
+    Q = rng.integers(0, 64, size=(14, 4)).astype(np.float32)
+    seeds = some[rng.integers(0, m, size=(14, 9))]
+    seeds[:, 4] = seeds[:, 1]
+    idx = onng.Index(_dev(ptr), _dev(col), _dev(X))
+    cta = 1024 + 4 * ((n + 8191) // 8192 * 1024 + 16384 * 4 + 16384 * 8)
+
+    class OneCta:
+        def get(self, need, device):
+            return torch.full((cta,), 0xA5, dtype=torch.uint8, device=device)
+    for k, e_s, eps, padded in ((10, 0, np.inf, 0), (10, 30, 0.3, 0), (40, 0, 0.1, 0), (10, 20, np.inf, 20), (5, 20, 0.2, 20)):
+        if padded:
+            idx.with_adjacency(padded)
+        for workspace in (None, OneCta()):
+            ids, dist, st = onng.search(idx, _dev(Q), k, e_s, eps, _dev(seeds), workspace=workspace)
+            o_ids, o_dist, o_st = oracle.search(ptr, col, X, Q, k, e_s, np.float32(eps), seeds)
+            assert np.array_equal(ids.cpu().numpy(), o_ids)
+            assert np.allclose(dist.cpu().numpy(), o_dist, rtol=1e-6)
+            assert np.array_equal(st[:, :2].cpu().numpy(), o_st[:, :2]) and (st[:, 3] == 0).all()
+
+
 @pytest.mark.parametrize("distinct", [1, 2, 5, 32])
 def test_repeated_seeds(distinct):
     """Seeds that repeat few ids over a whole batch and over several: each counts once."""

@@ -80,4 +80,18 @@ __device__ __forceinline__ unsigned long long pack_key(float d, int id)
     return (static_cast<unsigned long long>(__float_as_uint(d)) << 32) | static_cast<unsigned int>(id);
 }
 
+// Packed float32 arithmetic: each half rounds as the scalar instruction does.
+__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 }  // namespace onng

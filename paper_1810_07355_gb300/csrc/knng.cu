@@ -284,13 +284,6 @@ Shares plan_shares(int64_t nq, int64_t rows, int64_t tiles, int64_t slots, int g
 
 constexpr int kSweepSms = 152;  // SMs the sweeps are planned for
 
-__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b, unsigned long long c)
-{
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 // The float32 sweep.  RM rows x 8 columns per thread, so a row block is BM = 16 RM
 // rows: sweeps of fewer than 128 queries take the smallest block that holds them
 // (the arithmetic of padding rows is what bounded them).  The products use packed

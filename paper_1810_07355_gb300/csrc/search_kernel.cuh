@@ -300,20 +300,6 @@ __device__ __forceinline__ u64 pack_f32x2(float lo, float hi)
 }
 __device__ __forceinline__ float lo_f32(u64 v) { return __uint_as_float((unsigned)v); }
 __device__ __forceinline__ float hi_f32(u64 v) { return __uint_as_float((unsigned)(v >> 32)); }
-// packed float32 arithmetic: each half rounds as the scalar instruction does
-__device__ __forceinline__ u64 add_f32x2(u64 a, u64 b)
-{
-    u64 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ u64 fma_f32x2(u64 a, u64 b, u64 c)
-{
-    u64 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 static __device__ const float4 g_zero_quad = {0.f, 0.f, 0.f, 0.f};
 
 // A quad is 4 consecutive coordinates of a stored vector: read() its bytes, value()

@@ -103,19 +103,6 @@ struct PivSmem {
     unsigned long long best[kPivQ][kMaxSeed];
 };
 
-__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b)
-{
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b, unsigned long long c)
-{
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-
 // Inserts `key` (warp-uniform, absent from the list) into the ascending list
 // whose element e = h * 32 + lane is b[h] of lane `lane`; the last element drops.
 __device__ __forceinline__ void list_insert(unsigned long long (&b)[2], unsigned long long key, int lane)

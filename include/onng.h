@@ -135,8 +135,9 @@ int onng_adjust_degree_sac(const int32_t *nbr, const float *len, int64_t n, int3
 /* ------------------------------------------------------------ path adjustment
  * Algorithms 4/5 (AdjustPath / HasPath) read order-free: edge (i, j) is dropped
  * when the INPUT graph has i->m and m->j with len(i,m) < len(i,j) and
- * len(m,j) < len(i,j) (stored float32 lengths, strict comparisons).  Kept edges
- * keep their order.  Outputs: row_ptr_out [n+1]; col_out / len_out need room for
+ * len(m,j) < len(i,j) (stored float32 lengths, strict comparisons).  The row of a
+ * node that occurs in any list, and any row of more than 256 edges, is ordered by
+ * length (as the degree adjustment writes them).  Kept edges keep their order.  Outputs: row_ptr_out [n+1]; col_out / len_out need room for
  * the input edge count.  If nnz_host != NULL the call synchronises and stores
  * the kept edge count there.  removed_by (optional, [nnz_in] int32) receives, for
  * every input edge, the smallest-position witness m or -1.

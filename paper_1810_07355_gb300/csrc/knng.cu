@@ -1393,8 +1393,8 @@ __global__ void split_rows_kernel(const float *__restrict__ M, int64_t rows, int
 //   integer below 2^23): its 8-bit fields times 2^16, 2^8 and 1, each exact in
 //   bfloat16; zeros elsewhere.  The MMA then accumulates q.x - floor(|x|^2 / 2) exactly.
 //   Padding d to whole K atoms takes byte rows of any d = 32 .. 128 here from the float32
-//   sweep (30,011 x 100, the whole build: 20.5 -> 9.3 ms by this alone, 5.8 now); below
-//   32 the ties of small integers would flood the lists.
+//   sweep (30,011 x 100, the whole build: 20.5 -> 9.3 ms by this alone, 5.7 now); below
+//   32 a padded row would be mostly zeros, and the float32 sweep serves it.
 __global__ void prepare_rows_kernel(const float *__restrict__ M, int64_t rows, int d, int dpa, bool base,
                                     float *__restrict__ norm, __nv_bfloat16 *__restrict__ out, int *flag)
 {

@@ -38,7 +38,7 @@
 // the nearer of S's head and the batch's nearest member if that one will be
 // pushed (its distance is within the bound before the batch).  Its adjacency
 // row is loaded right then, so the load overlaps the R and S updates, and once
-// the row is in, its neighbours' vectors are prefetched into L2 (float32).
+// the row is in, its neighbours' vectors are prefetched into L2 (float32, d <= 256).
 //
 // Adjacency is read from the CSR lists, or from an optional padded table
 // adj [n, width] (-1 padded) that holds each node's first `width` entries, which
@@ -48,8 +48,9 @@
 // with keys inserted one at a time, one copy of the batch per call site, every bitmap
 // cleared before each search) and after, seeds included: 10,000 queries on 1M x 128
 // bfloat16 3.27 -> 2.83 ms, float32 4.85 -> 4.30 ms; 137 queries for 100 neighbours
-// 380 -> 285 us; word vectors whose candidates spill (200,000 x 100, 2,000 queries)
-// 41 -> 25 ms, of which most is refill_slow.
+// 380 -> 285 us.  A batch of word vectors takes as long as its slowest query's chain of
+// expansions: 200,000 x 100, 2,000 queries, 7 to 50 ms over five draws, 3,700 to 22,000
+// expansions of 3,900 to 4,600 cycles, refills of the head 9 to 25 % of them.
 //
 // Distances are squared float32 sums of (q - x)^2; the bound r^2 (1 + eps)^2 is
 // formed in double whenever r changes and kept rounded down to float32, which
@@ -85,11 +86,11 @@
 // (a power of two), shared-memory overflow keys per warp (128 or more, a power of
 // two), the most vector pairs gathered per round at d <= 128 (4 or 8) and the resident
 // CTAs per SM the registers are sized for.  What bounds the search is the instructions
-// and branches of an expansion (about 850 and 68 of them, each expansion waiting for the
-// one before) more than its bytes, so resident warps help only while a whole batch's
-// loads stay in registers: on 1M x 128, 10,000 queries, bfloat16 ran 2.84 ms at 5 CTAs,
-// 3.49 at 6 (spills), 3.05 at 4, and 2.97 with 4 pairs a round; float32 4.41 ms at 4
-// CTAs, 4.59 at 5, 5.21 at 3, and 4.78 with 4 pairs.
+// of an expansion (about 820 in float32 and 880 in bfloat16, 108 of them branches and
+// their kind, each expansion waiting for the one before) more than its bytes, so resident
+// warps help only while a whole batch's loads stay in registers: on 1M x 128, 10,000
+// queries, bfloat16 ran 2.84 ms at 5 CTAs, 3.49 at 6 (spills), 3.05 at 4, and 2.97 with 4
+// pairs a round; float32 4.41 ms at 4 CTAs, 4.59 at 5, 5.21 at 3, and 4.78 with 4 pairs.
 #ifndef ONNG_SEARCH_F32_HV
 #define ONNG_SEARCH_F32_HV 2048
 #endif
@@ -449,9 +450,9 @@ __device__ __noinline__ Levels make_room_slow(Levels s, u64 *ovf, u64 *gpool, in
 // passes over the pool.  In the first every lane keeps the 8 least of the keys it reads;
 // any key below the least of the lanes' 8th ones is among those kept, so the kept keys up
 // to that one (about 110 of a large pool) are its nearest.  The second drops what was
-// taken or is out of bound.  Both have several loads in flight: a query that lives in
-// the pool (word vectors: 10,000 candidates) spent four fifths of its time here when
-// each 128 keys were sorted into the best so far.
+// taken or is out of bound.  Both have several loads in flight, since one warp reads the
+// whole pool twice: a query of 22,000 expansions over word vectors came here 202 times
+// for a pool of 7,800 keys on average, a quarter of its cycles.
 template <int OVF> __device__ __noinline__ Levels refill_slow(Levels s, u64 *ovf, u64 *gpool, float bnd, int lane)
 {
     if (s.no == 0) {
